@@ -264,7 +264,7 @@ def prepare(case, seed):
     return st
 
 
-FALLBACK_STD = 0.12    # luminance spread above which a tile falls back: some 10 % of the tiles
+FALLBACK_STD = 0.06    # luminance spread above which a tile falls back: about 10 % of a 720p frame's tiles
 
 
 def run(st):
