@@ -35,6 +35,27 @@ namespace svgf {
 namespace dev {
 
 
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float lg2_approx(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Rec. 709 luma, Reinhard forward and inverse maps (Sec. 3.4).  Written as explicit fused
 // multiply-adds: every kernel that evaluates them then rounds identically (the compiler may not
 // contract a plain a * b + c the same way in two kernels).
@@ -86,21 +107,6 @@ __device__ __forceinline__ float2 depth_grad(const float4* __restrict__ g, int x
 __device__ __forceinline__ float2 depth_grad_interior(const float4* __restrict__ gp, int W) {
     return make_float2(0.5f * (__ldg(&gp[1].w) - __ldg(&gp[-1].w)),
                        0.5f * (__ldg(&gp[W].w) - __ldg(&gp[-W].w)));
-}
-
-// Natural log of the normal weight max(0, 1 - |a - b|^2 / 2)^sigma_n (-inf when it is 0).
-__device__ __forceinline__ float log_w_normal(float4 a, float4 b, float sigma_n) {
-    float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-    float t = 0.5f * fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    if (!(t < 1.0f)) return -INFINITY;
-    return sigma_n * log1pf(-t);
-}
-
-// Depth term of the log weight: |z_q - z_p| / (sigma_z |grad . offset| + eps).
-__device__ __forceinline__ float depth_term(float zp, float zq, float2 gr, float dx, float dy,
-                                            float sigma_z, float eps) {
-    float den = fmaf(sigma_z, fabsf(fmaf(gr.x, dx, gr.y * dy)), eps);
-    return __fdividef(fabsf(zq - zp), den);
 }
 
 __device__ __forceinline__ int start_level(const Params& P, const float* __restrict__ rough, long p) {
@@ -491,12 +497,59 @@ struct SpatialSmem {
     float2 m[kVarWindowPx];   // first two components of the moment record
 };
 
+// The weight of a spatial-variance tap is the a-trous weight without the luminance term, in natural
+// units and to full FP32 accuracy: a weighted variance magnifies a weight's relative error by up
+// to max (x - m)^2 / var, and log2-unit weights took it past 1e-5 of the exact value.
+
+// t = |n_p - n_q|^2 / 2 of the normal weight (1 - t)^sigma_n.
+__device__ __forceinline__ float normal_t(const float4& g, const float4& gq) {
+    const float ax = g.x - gq.x, ay = g.y - gq.y, az = g.z - gq.z;
+    return 0.5f * fmaf(ax, ax, fmaf(ay, ay, az * az));
+}
+
+// log(1 - t) where nearly every tap lies, t <= kNearT (normals less than 14 degrees apart): the
+// power series to t^5 (truncation below 5e-9 relative at 1/32).  Elsewhere log1pf, -inf for t >= 1
+// and for a t that is not a number.
+constexpr float kNearT = 0.03125f;
+__device__ __forceinline__ float log1m_near(float t) {
+    float p = fmaf(t, 1.0f / 5.0f, 1.0f / 4.0f);
+    p = fmaf(t, p, 1.0f / 3.0f);
+    p = fmaf(t, p, 0.5f);
+    return -fmaf(t, __fmul_rn(t, p), t);
+}
+__device__ __forceinline__ float log1m_far(float t) { return t < 1.0f ? log1pf(-t) : -INFINITY; }
+
+// exp(e) for e <= 0: 2^h with h = e log2 e rounded, times 1 + (residual of h) ln 2.
+__device__ __forceinline__ float exp_neg(float e) {
+    const float h = __fmul_rn(e, 1.4426950216293335f);   // log2 e to FP32, and its remainder below
+    const float r = fmaf(e, 1.925963e-8f, fmaf(e, 1.4426950216293335f, -h));
+    const float w = ex2_approx(h);
+    return fmaf(__fmul_rn(w, 0.6931471805599453f), r, w);
+}
+
+// The weight from l = log(1 - t): 0 where the normal weight is 0 or the weight is not a number.
+__device__ __forceinline__ float spatial_weight(const Params& P, float l, float zp, float zq, float2 gr,
+                                                float dx, float dy) {
+    const float den = fmaf(P.sigma_z, fabsf(fmaf(gr.x, dx, __fmul_rn(gr.y, dy))), P.eps);
+    const float depth = __fmul_rn(fabsf(zq - zp), rcp_approx(fmaxf(den, 1.17549435e-38f)));
+    const float w = exp_neg(fmaf(P.sigma_n, l, -depth));
+    return w > 0.f ? w : 0.f;
+}
+
 // The spatial variance of the pixels with a short history in the tile at (x0, y0) (a tile the
 // temporal stage flagged).  The block first copies the tile's window of G-buffer and moments to
 // shared memory (every load of the window in flight at once), then each short-history pixel
-// sums its (2R + 1)^2 taps from there, in the same order as a direct read.  Called by every
-// thread of the block (two barriers).  RC > 0 gives the radius as a constant (the loops are
-// unrolled); RC = 0 reads it from P.
+// sums its (2R + 1)^2 taps from there.  Called by every thread of the block (two barriers).
+//
+// E_w[mu2] - E_w[mu1]^2 = E_w[S] + Var_w[mu1], and Var_w[mu1] is formed without a difference of
+// large sums, so it keeps its FP32 accuracy for wide windows: RC > 0 (the radius as a constant)
+// takes the rows in a rolled loop, a row's mean and then its squared deviations from the weights
+// in registers, and merges the rows by Chan's pairwise update.  Bound by instruction issue (79 %
+// with every pixel short): about 52 instructions a tap, where the per-tap update with its
+// division, log1pf and expf took about 95, and a body of one row, where 49 unrolled taps did not
+// fit the instruction cache.  2560x1440 with every pixel short 556 -> 310 us, a steady 1080p
+// frame (some 50 flagged tiles) 21.4 -> 16.3 us.  RC = 0 (the radius from P) keeps West's per-tap
+// update.
 template <class S, int RC>
 __device__ __forceinline__ void spatial_variance_tile_r(const Params& P, int W, int H, int x0,
                                                         int y0, const float4* __restrict__ gbuf,
@@ -510,44 +563,90 @@ __device__ __forceinline__ void spatial_variance_tile_r(const Params& P, int W, 
     for (int i = threadIdx.y * TILE_X + threadIdx.x; i < HW * HH; i += TILE_X * TILE_Y) {
         const int yy = i / HW, xx = i - yy * HW;
         const int gx = x0 - R + xx, gy = y0 - R + yy;
+        // outside the image: a normal that is no number, whose weight is 0
+        float4 gq = make_float4(NAN, 0.f, 0.f, 0.f);
         if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
             const int q = gy * W + gx;
-            sm.g[i] = __ldg(&gbuf[q]);
+            gq = __ldg(&gbuf[q]);
             const float4 mq = S::ld_mom(mom, q);
             sm.m[i] = make_float2(mq.x, mq.y);
         }
+        sm.g[i] = gq;
     }
     __syncthreads();
     if (work) {
         const int c = (threadIdx.y + R) * HW + threadIdx.x + R;
         const float4 g = sm.g[c];
         const float2 gr = depth_grad(gbuf, x, y, W, H);
-        // E_w[mu2] - E_w[mu1]^2 = E_w[S] + Var_w[mu1].  Var_w[mu1] by West's weighted incremental
-        // update (running weighted mean and sum of squared deviations), which involves no
-        // difference of large sums and so keeps its FP32 accuracy for wide windows
         float sw = 0.f, sS = 0.f, mean = 0.f, m2 = 0.f;
+        if constexpr (RC > 0) {
+#pragma unroll 1
+            for (int b = -RC; b <= RC; ++b) {
+                if (y + b < 0 || y + b >= H) continue;
+                constexpr int N = 2 * RC + 1;
+                const int q0 = c + b * HW - RC;
+                float w[N], m[N], z[N];
+                bool far = false;
 #pragma unroll
-        for (int b = -R; b <= R; ++b) {
-            const int qy = y + b;
-            if (qy < 0 || qy >= H) continue;
+                for (int a = 0; a < N; ++a) {
+                    const float4 gq = sm.g[q0 + a];
+                    z[a] = gq.w;
+                    const float t = normal_t(g, gq);
+                    far = far || !(t <= kNearT);
+                    m[a] = t;
+                    w[a] = log1m_near(t);
+                }
+                if (far) {
 #pragma unroll
-            for (int a = -R; a <= R; ++a) {
-                const int qx = x + a;
-                if (qx < 0 || qx >= W) continue;
-                const int q = c + b * HW + a;
-                const float4 gq = sm.g[q];
-                const float e = log_w_normal(g, gq, P.sigma_n) -
-                                depth_term(g.w, gq.w, gr, (float)a, (float)b, P.sigma_z, P.eps);
-                const float w = expf(e);
-                if (!(w > 0.f)) continue;   // a zero weight changes nothing (and would give 0/0 first)
-                const float2 mq = sm.m[q];
-                const float t = sw + w;
-                const float d = mq.x - mean;
-                const float r = __fdividef(d * w, t);
-                m2 = fmaf(sw * d, r, m2);
-                mean += r;
+                    for (int a = 0; a < N; ++a)
+                        if (!(m[a] <= kNearT)) w[a] = log1m_far(m[a]);
+                }
+                float rw = 0.f, rm = 0.f;
+#pragma unroll
+                for (int a = 0; a < N; ++a) {
+                    w[a] = spatial_weight(P, w[a], g.w, z[a], gr, (float)(a - RC), (float)b);
+                    // a tap of weight 0 adds nothing, whatever its moments hold
+                    const float2 mq = w[a] > 0.f ? sm.m[q0 + a] : make_float2(0.f, 0.f);
+                    m[a] = mq.x;
+                    rw += w[a];
+                    rm = fmaf(w[a], mq.x, rm);
+                    sS = fmaf(w[a], mq.y, sS);
+                }
+                if (!(rw > 0.f)) continue;
+                const float row_mean = rm / rw;
+                float r2 = 0.f;
+#pragma unroll
+                for (int a = 0; a < N; ++a) {
+                    const float d = m[a] - row_mean;
+                    r2 = fmaf(w[a] * d, d, r2);
+                }
+                const float t = sw + rw, d = row_mean - mean, f = __fdiv_rn(rw, t);
+                m2 += fmaf(__fmul_rn(d, d), __fmul_rn(sw, f), r2);
+                mean = fmaf(d, f, mean);
                 sw = t;
-                sS = fmaf(w, mq.y, sS);
+            }
+        } else {
+#pragma unroll 1
+            for (int b = -R; b <= R; ++b) {
+                if (y + b < 0 || y + b >= H) continue;
+#pragma unroll 1
+                for (int a = -R; a <= R; ++a) {
+                    if (x + a < 0 || x + a >= W) continue;
+                    const int q = c + b * HW + a;
+                    const float4 gq = sm.g[q];
+                    const float tn = normal_t(g, gq);
+                    const float w = spatial_weight(P, tn <= kNearT ? log1m_near(tn) : log1m_far(tn), g.w, gq.w, gr,
+                                                   (float)a, (float)b);
+                    if (!(w > 0.f)) continue;   // a zero weight changes nothing (and would give 0/0 first)
+                    const float2 mq = sm.m[q];
+                    const float t = sw + w;
+                    const float d = mq.x - mean;
+                    const float r = __fdividef(d * w, t);
+                    m2 = fmaf(sw * d, r, m2);
+                    mean += r;
+                    sw = t;
+                    sS = fmaf(w, mq.y, sS);
+                }
             }
         }
         S::st_var(cv, p, fmaxf(0.f, sS / sw + m2 / sw));
@@ -582,27 +681,6 @@ __device__ __forceinline__ void spatial_variance_tile(const Params& P, int W, in
 //  - log2e is folded into the per-pixel constants.
 // Blocks whose tile lies at least two maximal steps inside the image take a path without
 // bounds checks (block-uniform branch).
-
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float lg2_approx(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float sqrt_approx(float x) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;

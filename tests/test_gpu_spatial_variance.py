@@ -1,0 +1,67 @@
+"""The 7x7 variance estimate of short histories where its weights change form: normals so close
+that log(1 - t) takes the power series, around the switch to log1pf at t = 1/32, far apart and
+opposed, in images smaller than the window and across tile edges.
+
+The reference is the estimate's definition in FP64, E_w[S] + Var_w[mu1] on a first frame (S = 0),
+with the variance formed from deviations: the oracle's difference of moments cancels to 0 where
+all but the centre's weight is below 1e-16, which these normals reach."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2312_06827_gb300 import svgf
+from parity import VAR_TOL
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24
+LUMA = np.array([0.2126, 0.7152, 0.0722])
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def first_frame_variance(luma, gbuf, sigma_z, sigma_n, eps, r=3):
+    h, w = luma.shape
+    z = gbuf[..., 3]
+    gx, gy = (np.gradient(z, axis=1) if w > 1 else 0 * z), (np.gradient(z, axis=0) if h > 1 else 0 * z)
+    out = np.zeros((h, w))
+    for y in range(h):
+        for x in range(w):
+            ys, xs = slice(max(0, y - r), y + r + 1), slice(max(0, x - r), x + r + 1)
+            dy, dx = np.mgrid[ys, xs][:, :h - ys.start, :w - xs.start] - np.array([y, x])[:, None, None]
+            q = gbuf[ys, xs]
+            t = np.minimum(0.5 * ((q[..., :3] - gbuf[y, x, :3]) ** 2).sum(-1), 1.0)
+            with np.errstate(divide="ignore"):
+                e = sigma_n * np.log1p(-t) - np.abs(q[..., 3] - z[y, x]) / (
+                    sigma_z * np.abs(gx[y, x] * dx + gy[y, x] * dy) + eps)
+            wt, m = np.exp(e), luma[ys, xs]
+            mean = (wt * m).sum() / wt.sum()
+            out[y, x] = (wt * (m - mean) ** 2).sum() / wt.sum()
+    return out
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (3, 9), (33, 8), (40, 21), (97, 35)])
+@pytest.mark.parametrize("spread", [0.02, 0.18, 1.5])
+@pytest.mark.parametrize("sigma_n", [2.0, 128.0])
+def test_weights_around_the_series_switch(w, h, spread, sigma_n):
+    rng = np.random.default_rng([w, h, int(100 * spread)])
+    n = np.array([0.0, 0.0, 1.0]) + spread * rng.standard_normal((h, w, 3))
+    n /= np.linalg.norm(n, axis=-1, keepdims=True)
+    z = 5.0 + 0.02 * np.arange(w)[None, :] + 0.01 * rng.standard_normal((h, w))
+    gbuf = np.concatenate([n, z[..., None]], -1).astype(np.float32)
+    noisy = rng.exponential(1.0, (h, w, 3)).astype(np.float32)
+    motion, rough = np.zeros((h, w, 2), np.float32), np.full((h, w), 0.5, np.float32)
+    cfg = svgf.default_config(w, h)
+    cfg.sigma_n = sigma_n
+    d = svgf.Denoiser(cfg)
+    cv = torch.empty(h, w, 4, device="cuda")
+    d.reproject_accumulate(svgf.make_frame(dev(noisy), dev(gbuf), dev(motion), dev(rough)), cv)
+    got = cv[..., 3].cpu().numpy().astype(np.float64)
+    l = noisy.astype(np.float64) @ LUMA
+    l = l / (1.0 + l)
+    ref = first_frame_variance(l, gbuf.astype(np.float64), cfg.sigma_z, sigma_n, float(np.float32(cfg.eps)))
+    # the stage's bar: 1e-5 of the value, and the rounding that FP32 luminances carry
+    tol = VAR_TOL * ref + 8 * U * l.max() * np.sqrt(ref)
+    assert np.all(np.abs(got - ref) <= tol), np.abs(got - ref).max()
