@@ -799,7 +799,7 @@ svgf_status batch_temporal(svgf_batch* b, int i0, int i1, const svgf_frame* fram
     memset(&ta, 0, sizeof ta);
     memset(&sa, 0, sizeof sa);
     ta.n = sa.n = i1 - i0;
-    int total = 0;
+    int total = 0, tiles_x[svgf::kMaxBatch];
     for (int i = i0; i < i1; ++i) {
         svgf_handle* h = b->hs[i];
         const svgf_frame* f = &frames[i];
@@ -834,6 +834,7 @@ svgf_status batch_temporal(svgf_batch* b, int i0, int i1, const svgf_frame* fram
         e.H = d.H;
         e.tiles_x = d.tiles_x;
         e.tile_base = total;
+        tiles_x[i - i0] = d.tiles_x;
         total += (int)(g.x * g.y);
     }
     ta.total = sa.total = total;
@@ -850,8 +851,10 @@ svgf_status batch_temporal(svgf_batch* b, int i0, int i1, const svgf_frame* fram
     }
     {
         LaunchScope L(h0, SVGF_K_SPATIAL_VAR, s);
-        svgf_status st = L.done(svgf::launch_batch_spatial(b->cfg.precision, sa,
-                                                           grid_for(total, b->sm_count, b->stage_bps), s));
+        // the resident grid of the single-frame launch: one block a tile (54,000 blocks for
+        // 14 Mpixel, nearly all of them finding their flag clear) cost more than the flagged tiles
+        svgf_status st = L.done(svgf::launch_batch_spatial(
+            b->cfg.precision, sa, svgf::spatial_grid(total, b->sm_count, tiles_x, i1 - i0), s));
         if (st != SVGF_OK) return st;
     }
     for (int i = i0; i < i1; ++i) {

@@ -50,7 +50,7 @@ kb_temporal(const __grid_constant__ BatchTemporalArgs A) {
 }
 
 template <class S, bool UP>
-__global__ void __launch_bounds__(TILE_X* TILE_Y)
+__global__ void __launch_bounds__(TILE_X* TILE_Y, kSpatialBlocksPerSM)
 kb_spatial_variance(const __grid_constant__ BatchSpatialArgs A) {
     // the flags of TILE_X * TILE_Y of the block's tiles are read at once, one per thread, and the
     // set ones collected in a shared bit mask (as in the single-frame kernel)

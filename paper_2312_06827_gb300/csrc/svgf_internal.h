@@ -52,6 +52,36 @@ inline dim3 atrous_grid(int mode, int iter, int W, int H) {
     return dim3((unsigned)((W + TILE_X - 1) / TILE_X), (unsigned)(((H + rows - 1) / rows) * ys));
 }
 
+// Resident blocks per SM of the spatial-variance grid (48 registers a thread).
+constexpr int kSpatialBlocksPerSM = 5;
+
+// Grid of the spatial-variance launch over n_tiles tiles: the resident blocks, which read the flags
+// of their tiles t = b, b + grid, ... 256 at a time, so that the few flagged tiles of a
+// steady-state frame cost one flag load each for the rest and not a block launch.  Kept coprime
+// with the tile row lengths (tiles_x of the n images): a column of flagged tiles (the image edge a
+// camera pan uncovers) then lands on as many blocks as it has tiles instead of on grid / gcd of
+// them, where they would run one after another.
+inline int spatial_grid(int n_tiles, int sms, const int* tiles_x, int n) {
+    int grid = n_tiles < sms * kSpatialBlocksPerSM ? n_tiles : sms * kSpatialBlocksPerSM;
+    auto gcd = [](int a, int b) {
+        while (b) {
+            const int r = a % b;
+            a = b;
+            b = r;
+        }
+        return a;
+    };
+    for (int i = 0; i < n && grid > 1;) {
+        if (gcd(grid, tiles_x[i]) == 1) {
+            ++i;
+        } else {
+            --grid;
+            i = 0;
+        }
+    }
+    return grid;
+}
+
 // Bytes per pixel of a workspace image (colour + variance, colour history, moments) in each
 // storage precision (svgf_config.precision): float4, or an 8-byte 16-bit record.
 inline size_t image_bytes_per_px(int prec) { return prec == 0 ? 16 : 8; }

@@ -32,9 +32,6 @@ k_temporal(Params P, const float* __restrict__ noisy, const float4* __restrict__
                      hist_prev, mom_prev, has_history, cv_out, mom_out, hist_accum_out, sm);
 }
 
-// Resident blocks per SM of the spatial-variance grid (32 registers a thread).
-constexpr int kSpatialBlocksPerSM = 5;
-
 // A resident grid walks the tiles t = blockIdx.x + k gridDim.x: the block reads the flags of
 // TILE_X * TILE_Y such tiles at once (one per thread), gathers the set ones in a shared bit mask
 // and runs the tile kernel on each.  In a steady-state frame few tiles are flagged, and the rest
@@ -211,22 +208,10 @@ cudaError_t launch_spatial_variance(int prec, const Params& P, const float4* gbu
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    int grid = n_tiles < sms * kSpatialBlocksPerSM ? n_tiles : sms * kSpatialBlocksPerSM;
-    // Block b takes tiles b, b + grid, ...: with grid and the tile row length coprime, a column of
-    // flagged tiles (the image edge a camera pan uncovers) lands on as many blocks as it has
-    // tiles instead of on grid / gcd of them, where they would run one after another.
-    auto gcd = [](int a, int b) {
-        while (b) {
-            const int r = a % b;
-            a = b;
-            b = r;
-        }
-        return a;
-    };
-    while (grid > 1 && gcd(grid, (int)tiles.x) != 1) --grid;
+    const int tiles_x = (int)tiles.x, grid = spatial_grid(n_tiles, sms, &tiles_x, 1);
 #define SVGF_SPATIAL(ST)                                                                        \
     k_spatial_variance<ST><<<grid, block, 0, s>>>(P, gbuf, (const ST::Rec*)mom, tile_flags, n_tiles, \
-                                                   (int)tiles.x, (ST::Rec*)cv)
+                                                   tiles_x, (ST::Rec*)cv)
     switch (prec) {
         case 0: SVGF_SPATIAL(StoreF32); break;
         case 1: SVGF_SPATIAL(Store16<false>); break;
