@@ -4,8 +4,8 @@
 //   conv x4   3x3, 10 -> 32 -> 32 -> 32 -> 25 (ReLU between), BF16 operands, FP32 accumulation,
 //             as implicit GEMMs on the 5th-generation tensor cores (tcgen05.mma, accumulators in
 //             tensor memory); the same kernel computes the data gradient (dgrad) with the
-//             flipped, transposed weights; the weight gradient (wgrad) is a second tensor-core
-//             GEMM reduced over pixels (mma.sync m16n8k16 bf16, ldmatrix from padded tiles)
+//             flipped, transposed weights; the weight gradient (wgrad) is a second tcgen05
+//             GEMM, reduced over pixels
 //   apply     softmax of the 25 logits = a 5x5 kernel per pixel (computed in the last layer's
 //             epilogue, stored as 25 planes), applied to the pass-0 colour at dilation 1 and then
 //             at dilation 4 (renormalised over in-image taps)
@@ -30,27 +30,8 @@ namespace svgf {
 namespace kpn {
 namespace {
 
-constexpr int TX = 16, TY = 8;        // conv output tile: 8 rows x 16 pixels, one row per warp
-
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void ldsm_x4_t(unsigned& r0, unsigned& r1, unsigned& r2, unsigned& r3,
-                                          const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(smem_addr(p)));
-}
-
-// D = A (16x16, row) * B (16x8, col) + D, BF16 operands, FP32 accumulators.
-__device__ __forceinline__ void mma_bf16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2,
-                                         unsigned a3, unsigned b0, unsigned b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-        "{%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
 __device__ __forceinline__ float ex2_fast(float x) {
@@ -69,23 +50,6 @@ __device__ __forceinline__ unsigned pack_f16(float lo, float hi) {
 }
 __device__ __forceinline__ float2 unpack_f16(unsigned u) {
     return __half22float2(*reinterpret_cast<const __half2*>(&u));
-}
-
-// Copy a (TY+2) x (TX+2) halo tile of a [B][H][W][CI] BF16 image into shared memory (pixel
-// stride CIP = CI + 8 to spread ldmatrix rows over the banks); zeros outside the image.
-template <int CI, int CIP>
-__device__ __forceinline__ void load_halo(__nv_bfloat16 (*s)[TX + 2][CIP], const __nv_bfloat16* in,
-                                          int n, int H, int W, int x0, int y0, int tid, int nthr) {
-    constexpr int CH = CI / 8;   // 16-byte chunks per pixel
-    for (int i = tid; i < (TY + 2) * (TX + 2) * CH; i += nthr) {
-        const int c = i % CH, px = i / CH;
-        const int ly = px / (TX + 2), lx = px - ly * (TX + 2);
-        const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (gx >= 0 && gy >= 0 && gx < W && gy < H)
-            v = *reinterpret_cast<const uint4*>(in + (((long)n * H + gy) * W + gx) * CI + c * 8);
-        *reinterpret_cast<uint4*>(&s[ly][lx][c * 8]) = v;
-    }
 }
 
 // ---- the 3x3 convolution on the 5th-generation tensor cores (tcgen05) ------------------------
@@ -1338,91 +1302,276 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_kpn_pair(const __nv_bfloat1
     if (warp == 0) tmem_dealloc(tmem, 2 * 32 * kPairSlots);
 }
 
-// Weight gradient of one layer: dW[co][tap][ci] += sum_p dZ[p][co] X[p + off(tap)][ci], over
-// co < CO_REAL, ci < CI_REAL (the padded channels carry no parameters).  Nine warps, one tap each;
-// every block walks tiles with a grid stride, keeps its partial sums in registers and adds them
-// to dW once at the end.
+// Weight and bias gradient of one layer: dW[co][tap][ci] += sum_p dZ[p][co] X[p + off(tap)][ci] and
+// db[co] += sum_p dZ[p][co], over co < co_real, ci < ci_real (the padded channels carry no
+// parameters), on the tensor cores (tcgen05).  The reduction runs over pixels, so both operands
+// are read MN-major straight from the staged rows: 16 pixels of an X row are K, and M = 128 covers
+// (dx, ci) because the descriptor's stride between channel groups is one pixel (the groups past
+// dx = 2 are not used).  N = 96 covers (dy, co): the three dZ rows that X row r meets, r - 1, r and
+// r + 1, which carry dy = 2, 1, 0.  One product of 16 pixels is thus 9 x 32 x CI of the gradient's
+// sums, and they stay in tensor memory over all of a block's rows (in kWgSets interleaved sets,
+// so that a sum's chain of additions stays short).
+//
+// A block walks chunks of X rows down one 128-pixel column of an image (two blocks a SM):
+//   warp 5, the producer: X rows (130 pixels) and dZ rows (128) into two rings by TMA, zeros
+//     outside the image from the tensor maps; dZ runs one row ahead and behind the chunk;
+//   warp 4, the issuer (the whole warp walks the rows, one elected lane issues);
+//   warps 0-3: the bias sums, from each staged dZ row of the chunk (a pixel a thread, its 32 sums
+//     in registers), and at the end the accumulators, one atomic add an entry and block.
+// They meet at mbarriers, waited for phase by phase as in k_conv3x3_tc: fullX / fullD (the row
+// landed) -> issuer, bias warps; freeX (commit) and freeD (commit of the last X row that meets it,
+// and one arrival a bias warp) -> the producer.  Slots follow running counts.
+// 16 crops of 256 x 256, 32 -> 32 channels: 124 + 26 us (mma.sync and a
+// separate bias sum) -> 40 us; layer 0, 10 -> 32 channels, 102 + 26 -> 39 us.  The products take 12
+// us of that and the operands' bytes 20 us of HBM; the rest is the row hand-offs and the blocks'
+// start and end.
+constexpr int kWgXRing = 4, kWgDRing = 6;
+constexpr unsigned kWgSets = 2;
+constexpr int kWgThreads = 192;
+constexpr int kWgDRow = tc::M * 64;                  // a staged dZ row: 128 pixels x 32 channels
 template <int CI>
-__global__ void __launch_bounds__(288) k_wgrad(const __nv_bfloat16* __restrict__ X,
-                                               const __nv_bfloat16* __restrict__ dZ, float* dW,
-                                               int B, int H, int W, int ci_real, int co_real) {
-    constexpr int CIP = CI + 8, NT = CI / 8;
-    __shared__ __align__(16) __nv_bfloat16 s_x[TY + 2][TX + 2][CIP];
-    __shared__ __align__(16) __nv_bfloat16 s_dz[TY][TX][40];
-    const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
-    const int dy = tap / 3, dx = tap % 3;
-    const int tiles_x = (W + TX - 1) / TX, tiles_y = (H + TY - 1) / TY;
-    const int total = tiles_x * tiles_y * B;
-    float acc[2][NT][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < NT; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-    const int mi = lane >> 3, ri = lane & 7;
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const int n = t / (tiles_x * tiles_y), r = t - n * tiles_x * tiles_y;
-        const int y0 = (r / tiles_x) * TY, x0 = (r % tiles_x) * TX;
-        __syncthreads();
-        load_halo<CI, CIP>(s_x, X, n, H, W, x0, y0, tid, 288);
-        for (int i = tid; i < TY * TX * 4; i += 288) {
-            const int c = i & 3, px = i >> 2, ly = px / TX, lx = px % TX;
-            const int gx = x0 + lx, gy = y0 + ly;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);   // pixels outside the image contribute nothing
-            if (gx < W && gy < H)
-                v = *reinterpret_cast<const uint4*>(dZ + (((long)n * H + gy) * W + gx) * 32 + c * 8);
-            *reinterpret_cast<uint4*>(&s_dz[ly][lx][c * 8]) = v;
+struct WgradCfg {
+    static constexpr int XROW = CI == 32 ? kRowSw64Bytes : kRowSw32Bytes;
+    static constexpr int OFF_D = kWgXRing * XROW;
+    static constexpr int OFF_BIAS = OFF_D + kWgDRing * kWgDRow;      // [4][32] floats
+    static constexpr int OFF_BAR = OFF_BIAS + 4 * 32 * 4;
+    static constexpr int BARS = 2 * kWgXRing + 2 * kWgDRing + 1;
+    static constexpr int SMEM = OFF_BAR + BARS * 8 + 8;
+    static_assert(OFF_D % 512 == 0 && kWgDRow % 512 == 0, "row slots on swizzle boundaries");
+};
+
+template <int CI>
+__global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const __grid_constant__ CUtensorMap xmap,
+                                                         const __grid_constant__ CUtensorMap dmap, float* dW, float* db,
+                                                         int B, int H, int W, int chunk, int ci_real, int co_real,
+                                                         int* err) {
+    using namespace tc;
+    using Cfg = WgradCfg<CI>;
+    constexpr int RB = CI * 2;
+    extern __shared__ __align__(1024) unsigned char wg_smem[];
+    unsigned char *sx = wg_smem, *sd = wg_smem + Cfg::OFF_D;
+    float* sbias = reinterpret_cast<float*>(wg_smem + Cfg::OFF_BIAS);
+    uint64_t* full_x = reinterpret_cast<uint64_t*>(wg_smem + Cfg::OFF_BAR);
+    uint64_t *free_x = full_x + kWgXRing, *full_d = free_x + kWgXRing, *free_d = full_d + kWgDRing;
+    uint64_t* fin = free_d + kWgDRing;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(fin + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int i = 0; i < kWgXRing; ++i) {
+            mbar_init(&full_x[i]);
+            mbar_init(&free_x[i]);
         }
-        __syncthreads();
+        for (int i = 0; i < kWgDRing; ++i) {
+            mbar_init(&full_d[i]);
+            mbar_init(&free_d[i], 1 + 4);
+        }
+        mbar_init(fin);
+    }
+    if (warp == 0) tmem_alloc(tslot, 128 * kWgSets);
+    fence_proxy_async();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tslot;
+    if (warp < 4) {                                  // every sum starts at zero
 #pragma unroll 1
-        for (int row = 0; row < TY; ++row) {            // k chunk: the 16 pixels of one row
-            unsigned a[2][4];
+        for (unsigned c = 0; c < 128 * kWgSets; c += 32) st32_zero(tmem + c + ((uint32_t)(warp * 32) << 16));
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const int segs = (W + M - 1) / M, chunks_y = (H + chunk - 1) / chunk;
+    const long total = (long)B * segs * chunks_y;
+    struct Chunk {
+        int n, x0, y0, rows;
+    };
+    auto chunk_of = [&](long c) {
+        Chunk k;
+        k.n = (int)(c / ((long)segs * chunks_y));
+        const int rc = (int)(c - (long)k.n * segs * chunks_y), seg = rc / chunks_y;
+        k.x0 = seg * M;
+        k.y0 = (rc - seg * chunks_y) * chunk;
+        k.rows = (k.y0 + chunk < H ? k.y0 + chunk : H) - k.y0;
+        return k;
+    };
+
+    if (warp == 5) {
+        // ---- the producer
+        constexpr uint32_t kXTx = (uint32_t)HP * RB, kDTx = (uint32_t)kWgDRow;
+        unsigned nx = 0, nd = 0;                     // rows staged so far
+        uint32_t usedx = 0, usedd = 0, px = 0, pd = 0;   // per slot: used before, parity of its next free phase
+        uint32_t fx = 0, fd = 0;                     // per slot: parity of the next copy's phase
+        bool ok = true;
+        auto stage_x = [&](const Chunk& k, int row) {
+            const int sl = (int)(nx++ % kWgXRing);
+            if ((usedx >> sl) & 1u) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&free_x[sl], (px >> sl) & 1u));
+                px ^= 1u << sl;
+                if (!ok) return;
+            }
+            usedx |= 1u << sl;
+            fx ^= 1u << sl;
+            if (lane == 0) {
+                mbar_arrive_expect_tx(&full_x[sl], kXTx);
+                tma_load_4d(sx + sl * Cfg::XROW, &xmap, 0, k.x0 - 1, row, k.n, &full_x[sl]);
+            }
+            __syncwarp();
+        };
+        auto stage_d = [&](const Chunk& k, int row) {
+            const int sl = (int)(nd++ % kWgDRing);
+            if ((usedd >> sl) & 1u) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&free_d[sl], (pd >> sl) & 1u));
+                pd ^= 1u << sl;
+                if (!ok) return;
+            }
+            usedd |= 1u << sl;
+            fd ^= 1u << sl;
+            if (lane == 0) {
+                mbar_arrive_expect_tx(&full_d[sl], kDTx);
+                tma_load_4d(sd + sl * kWgDRow, &dmap, 0, k.x0, row, k.n, &full_d[sl]);
+            }
+            __syncwarp();
+        };
+        for (long c = blockIdx.x; c < total && ok; c += gridDim.x) {
+            const Chunk k = chunk_of(c);
+            stage_d(k, k.y0 - 1);
+            if (ok) stage_d(k, k.y0);
+            for (int i = 0; i < k.rows && ok; ++i) {
+                stage_x(k, k.y0 + i);
+                if (ok) stage_d(k, k.y0 + i + 1);
+            }
+        }
+        // the block's shared memory is released at its end: every copy issued must have landed
+        for (int sl = 0; sl < kWgXRing; ++sl)
+            if ((usedx >> sl) & 1u) mbar_wait(&full_x[sl], ((fx >> sl) & 1u) ^ 1u);
+        for (int sl = 0; sl < kWgDRing; ++sl)
+            if ((usedd >> sl) & 1u) mbar_wait(&full_d[sl], ((fd >> sl) & 1u) ^ 1u);
+        if (!ok && lane == 0) atomicOr(err, kErrWaitGaveUp);
+    } else if (warp == 4) {
+        // ---- the issuer: both operands MN-major (descriptor bits 15 and 16).  A: channel groups of
+        // one pixel's CI channels, one pixel apart (LBO), 8-pixel groups along K (SBO).  B: one dZ
+        // row's 32 channels a group, rows a slot apart.
+        const uint32_t mn = (1u << 15) | (1u << 16);
+        const uint64_t A0 = sdesc(smem_addr(sx), RB, 8 * RB) | ((CI == 32 ? 4ull : 6ull) << 61);
+        const uint64_t B0 = sdesc(smem_addr(sd), kWgDRow, 512) | (4ull << 61);
+        unsigned nx = 0, nd = 0;                     // X rows issued; dZ row i = 0 of the chunk
+        uint32_t px = 0, pd = 0;                     // per slot: parity of the next full phase
+        bool ok = true, any = false;
+        for (long c = blockIdx.x; c < total && ok; c += gridDim.x) {
+            const Chunk k = chunk_of(c);
+            const int kcs = ((W - k.x0 < M ? W - k.x0 : M) + 15) / 16;   // 16-pixel products a row
+            for (int i = 0; i < k.rows && ok; ++i) {
+                // dZ rows i .. i + 2 of the chunk meet X row i; the first X row waits for three
+                for (int j = i == 0 ? 0 : 2; j <= 2 && ok; ++j) {
+                    const int sl = (int)((nd + i + j) % kWgDRing);
+                    ok = __all_sync(0xffffffffu, mbar_wait(&full_d[sl], (pd >> sl) & 1u));
+                    pd ^= 1u << sl;
+                }
+                const int sl = (int)(nx % kWgXRing);
+                if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&full_x[sl], (px >> sl) & 1u));
+                px ^= 1u << sl;
+                if (!ok) break;
+                fence_after();
+                const int s0 = (int)((nd + i) % kWgDRing), first = kWgDRing - s0 < 3 ? kWgDRing - s0 : 3;
+                const uint32_t id1 = idesc_n(32u * first) | mn, id2 = idesc_n(32u * (3 - first)) | mn;
+                const uint32_t acc = tmem + (nx % kWgSets) * 128u;
+                for (int kc = 0; kc < kcs; ++kc) {
+                    const uint64_t a = A0 + (uint64_t)((sl * Cfg::XROW + kc * 16 * RB) >> 4);
+                    mma_elect(acc, a, B0 + (uint64_t)((s0 * kWgDRow + kc * 16 * 64) >> 4), id1);
+                    if (first < 3) mma_elect(acc + 32u * first, a, B0 + (uint64_t)((kc * 16 * 64) >> 4), id2);
+                }
+                any = true;
+                commit_elect(&free_x[sl]);
+                commit_elect(&free_d[s0]);
+                if (i == k.rows - 1) {               // the chunk's last two dZ rows are done too
+                    commit_elect(&free_d[(nd + i + 1) % kWgDRing]);
+                    commit_elect(&free_d[(nd + i + 2) % kWgDRing]);
+                }
+                ++nx;
+            }
+            nd += (unsigned)k.rows + 2;
+        }
+        if (!ok && lane == 0) atomicOr(err, kErrWaitGaveUp);
+        // the sums are read and the tensor memory freed below: every MMA must have completed
+        if (any) {
+            commit_elect(fin);
+            mbar_wait(fin, 0u);
+        }
+        __syncwarp();
+    } else {
+        // ---- the bias sums: thread t adds up pixel t of every dZ row of its chunks
+        float bs[32];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)              // A = dZ^T: rows co, k pixels
-                ldsm_x4_t(a[mt][0], a[mt][1], a[mt][2], a[mt][3],
-                          &s_dz[row][ri + ((mi & 2) ? 8 : 0)][mt * 16 + ((mi & 1) ? 8 : 0)]);
+        for (int j = 0; j < 32; ++j) bs[j] = 0.f;
+        unsigned nd = 0;
+        uint32_t pd = 0;
+        bool ok = true;
+        for (long c = blockIdx.x; c < total && ok; c += gridDim.x) {
+            const Chunk k = chunk_of(c);
+            for (int j = 0; j < k.rows + 2; ++j, ++nd) {
+                const int sl = (int)(nd % kWgDRing);
+                ok = __all_sync(0xffffffffu, mbar_wait(&full_d[sl], (pd >> sl) & 1u));
+                pd ^= 1u << sl;
+                if (!ok) break;
+                if (j >= 1 && j <= k.rows) {         // the halo rows belong to the neighbouring chunks
+                    const unsigned char* row = sd + sl * kWgDRow + tid * 64;
 #pragma unroll
-            for (int np = 0; np < NT / 2; ++np) {       // B = shifted X: k pixels, n inputs
-                unsigned b0, b1, b2, b3;
-                ldsm_x4_t(b0, b1, b2, b3,
-                          &s_x[row + dy][ri + ((mi & 1) ? 8 : 0) + dx][np * 16 + ((mi & 2) ? 8 : 0)]);
+                    for (int q = 0; q < 4; ++q) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(row + ((q ^ ((tid >> 1) & 3)) << 4));
+                        const unsigned u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                    mma_bf16(acc[mt][2 * np], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-                    mma_bf16(acc[mt][2 * np + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
+                        for (int h = 0; h < 4; ++h) {
+                            bs[8 * q + 2 * h] += __uint_as_float(u[h] << 16);
+                            bs[8 * q + 2 * h + 1] += __uint_as_float(u[h] & 0xffff0000u);
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&free_d[sl]);
+            }
+        }
+        if (!ok && lane == 0) atomicOr(err, kErrWaitGaveUp);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            float v = bs[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) sbias[warp * 32 + j] = v;
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp < 4) {
+        // accumulator lane = (dx, ci), column = (2 - dy, co)
+        if (tid < co_real) atomicAdd(&db[tid], (sbias[tid] + sbias[32 + tid]) + (sbias[64 + tid] + sbias[96 + tid]));
+        const int m = warp * 32 + lane, dx = m / CI, ci = m % CI;
+        if (warp * 32 < 3 * CI) {
+#pragma unroll 1
+            for (int blk = 0; blk < 3; ++blk) {
+                float sum[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) sum[j] = 0.f;
+#pragma unroll 1
+                for (unsigned st = 0; st < kWgSets; ++st) {
+                    uint32_t v[32];
+                    ld32(v, tmem + st * 128u + blk * 32u + ((uint32_t)(warp * 32) << 16));
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) sum[j] += __uint_as_float(v[j]);
+                }
+                if (dx < 3 && ci < ci_real) {
+                    const int tap = (2 - blk) * 3 + dx;
+#pragma unroll
+                    for (int co = 0; co < 32; ++co)
+                        if (co < co_real) atomicAdd(&dW[((long)co * 9 + tap) * ci_real + ci], sum[co]);
                 }
             }
         }
     }
-    const int g = lane >> 2, tq = lane & 3;
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int co = mt * 16 + g + ((e & 2) ? 8 : 0), ci = nt * 8 + 2 * tq + (e & 1);
-                if (co < co_real && ci < ci_real)
-                    atomicAdd(&dW[((long)co * 9 + tap) * ci_real + ci], acc[mt][nt][e]);
-            }
-}
-
-// Bias gradient: db[co] += sum_p dZ[p][co] (co < co_real).
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ dZ, float* db, long npx, int co_real) {
-    const int co = threadIdx.x & 31;
-    float s = 0.f;
-    for (long p = blockIdx.x * (long)(blockDim.x / 32) + (threadIdx.x >> 5); p < npx;
-         p += (long)gridDim.x * (blockDim.x / 32))
-        s += __bfloat162float(dZ[p * 32 + co]);
-    __shared__ float red[8][32];
-    red[threadIdx.x >> 5][co] = s;
+    fence_before();
     __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = 0.f;
-        for (int w = 0; w < (int)(blockDim.x / 32); ++w) v += red[w][co];
-        if (co < co_real) atomicAdd(&db[co], v);
-    }
+    fence_after();
+    if (warp == 0) tmem_dealloc(tmem, 128 * kWgSets);
 }
 
 // ---------------------------------------------------------------- softmax + kernel application
@@ -1795,10 +1944,10 @@ static int conv_chunk(int B, int H, int W, int sm_count) {
 }
 
 // The tensor map of a convolution's input [B][H][W][CI] BF16 for the producer's row copies: box
-// CI channels x 130 pixels x 1 row x 1 image, in the swizzle the MMAs read (64-byte rows for 32
+// CI channels x px pixels (130: a row with its halo) x 1 row x 1 image, in the swizzle the MMAs read (64-byte rows for 32
 // channels, 32-byte rows for 16), zeros outside the tensor.  cuTensorMapEncodeTiled is reached
 // through the runtime's driver entry point.
-static cudaError_t encode_rows(CUtensorMap* map, const __nv_bfloat16* in, int CI, int B, int H, int W) {
+static cudaError_t encode_rows(CUtensorMap* map, const __nv_bfloat16* in, int CI, int B, int H, int W, int px = tc::HP) {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     if (!fn) {
         void* p = nullptr;
@@ -1810,7 +1959,7 @@ static cudaError_t encode_rows(CUtensorMap* map, const __nv_bfloat16* in, int CI
     }
     const cuuint64_t dims[4] = {(cuuint64_t)CI, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[3] = {(cuuint64_t)CI * 2, (cuuint64_t)W * CI * 2, (cuuint64_t)H * W * CI * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)CI, (cuuint32_t)tc::HP, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)CI, (cuuint32_t)px, 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)in, dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CI == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
@@ -1904,18 +2053,22 @@ cudaError_t net_pairs(const __nv_bfloat16* feats, const WeightPtrs& w, __nv_bflo
 }
 
 cudaError_t wgrad(int layer, const __nv_bfloat16* X, const __nv_bfloat16* dZ, float* grad_flat,
-                  int B, int H, int W, int sm_count, cudaStream_t s) {
-    const int tiles = ((W + TX - 1) / TX) * ((H + TY - 1) / TY) * B;
-    const int grid = tiles < sm_count * 2 ? tiles : sm_count * 2;
+                  int B, int H, int W, int sm_count, cudaStream_t s, int* err) {
+    const int chunk = conv_chunk(B, H, W, sm_count);
+    const long tiles = (long)B * ((W + tc::M - 1) / tc::M) * ((H + chunk - 1) / chunk), cap = (long)sm_count * 2;
+    const int grid = (int)(tiles < cap ? tiles : cap);
     float* dW = grad_flat + param_offset(layer);
     float* db = dW + cout_of(layer) * 9 * cin_of(layer);
-    if (layer == 0) k_wgrad<16><<<grid, 288, 0, s>>>(X, dZ, dW, B, H, W, cin_of(0), cout_of(0));
-    else k_wgrad<32><<<grid, 288, 0, s>>>(X, dZ, dW, B, H, W, cin_of(layer), cout_of(layer));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long npx = (long)B * H * W;
-    k_bias_grad<<<flat_grid(npx, 256), 256, 0, s>>>(dZ, db, npx, cout_of(layer));
-    return cudaGetLastError();
+    auto launch = [&](auto kernel, int ci, int smem) {
+        CUtensorMap xmap, dmap;
+        cudaError_t e = encode_rows(&xmap, X, ci, B, H, W);
+        if (e == cudaSuccess) e = encode_rows(&dmap, dZ, 32, B, H, W, tc::M);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, kWgThreads, smem, s>>>(xmap, dmap, dW, db, B, H, W, chunk, cin_of(layer), cout_of(layer), err);
+        return cudaGetLastError();
+    };
+    return layer == 0 ? launch(k_wgrad<16>, 16, WgradCfg<16>::SMEM) : launch(k_wgrad<32>, 32, WgradCfg<32>::SMEM);
 }
 
 cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W,

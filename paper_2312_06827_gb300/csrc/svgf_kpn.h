@@ -55,9 +55,9 @@ cudaError_t net_pairs(const __nv_bfloat16* feats, const WeightPtrs& w, __nv_bflo
 // phase that nothing completes, gives up after `tries` polls and raises kErrWaitGaveUp in *err
 // the way a convolution block does.  Nothing else is touched.
 cudaError_t wait_expiry_probe(int tries, int* err, cudaStream_t s);
-// Adds the layer's weight and bias gradients into grad_flat (flat parameter layout).
+// Adds the layer's weight and bias gradients into grad_flat (flat parameter layout).  Waits as in conv.
 cudaError_t wgrad(int layer, const __nv_bfloat16* X, const __nv_bfloat16* dZ, float* grad_flat,
-                  int B, int H, int W, int sm_count, cudaStream_t s);
+                  int B, int H, int W, int sm_count, cudaStream_t s, int* err);
 // c_out = K-weighted mean of c_in at the given dilation (K planar [25][B*H*W]); with rgb_out, the
 // inverse tone map is fused and rgb_out.w = var_src.w.
 cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W,
