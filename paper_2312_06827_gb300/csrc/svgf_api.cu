@@ -1156,7 +1156,7 @@ struct svgf_kpn {
     svgf::kpn::WeightPtrs w;
     // workspace images (max_px pixels each)
     __nv_bfloat16 *x1, *x2, *x3, *dzA, *dzB, *feats;
-    float *K, *gK, *loss_sum;   // K, gK: 25 planes [25][pixels]
+    float *K, *loss_sum;         // K: 25 planes [25][pixels]
     float4 *c0, *c1, *c2, *u;
     unsigned char* tile_masks;   // kMaskArrays arrays of mask_stride bytes (one per 32x32 tile)
     size_t mask_stride;
@@ -1186,7 +1186,7 @@ size_t kpn_layout(int max_px, svgf_kpn* k) {
     const size_t o_b0 = take(128), o_b1 = take(128), o_b2 = take(128), o_b3 = take(128);
     const size_t o_x1 = take(n * 64), o_x2 = take(n * 64), o_x3 = take(n * 64);
     const size_t o_dzA = take(n * 64), o_dzB = take(n * 64), o_feats = take(n * 32);
-    const size_t o_K = take(n * 100), o_gK = take(n * 100);
+    const size_t o_K = take(n * 100);
     const size_t o_c0 = take(n * 16), o_c1 = take(n * 16), o_c2 = take(n * 16), o_u = take(n * 16);
     // 32x32 tiles of a frame of n pixels, each side <= 32768: at most n/1024 + 2048 + 1; the
     // fallback's tile masks: the flagged tiles and, per plain pass, the tiles it computes
@@ -1213,7 +1213,6 @@ size_t kpn_layout(int max_px, svgf_kpn* k) {
         k->dzB = (__nv_bfloat16*)(b + o_dzB);
         k->feats = (__nv_bfloat16*)(b + o_feats);
         k->K = (float*)(b + o_K);
-        k->gK = (float*)(b + o_gK);
         k->c0 = (float4*)(b + o_c0);
         k->c1 = (float4*)(b + o_c1);
         k->c2 = (float4*)(b + o_c2);
@@ -1247,19 +1246,18 @@ cudaError_t kpn_zero_err(svgf_kpn* k, cudaStream_t s) {
     return e;
 }
 
-// Forward through the four layers and the two applications (K and c1 kept for backward).
-cudaError_t kpn_run_forward(svgf_kpn* k, const __nv_bfloat16* feats, const float4* c0, int B, int H,
-                            int W, float4* c2, cudaStream_t s) {
+// Forward through the four layers and the two applications (K, c1 and c2 kept for backward); with
+// a target T also the squared error into loss_sum and u.
+cudaError_t kpn_run_forward(svgf_kpn* k, const __nv_bfloat16* feats, const float4* c0, const float4* T, int B,
+                            int H, int W, float4* c2, cudaStream_t s) {
     using namespace svgf::kpn;
     cudaError_t e = kpn_zero_err(k, s);
     if (e == cudaSuccess) e = conv(0, false, feats, k->w, nullptr, k->x1, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess) e = conv(3, false, k->x3, k->w, nullptr, k->K, B, H, W, k->sm_count, s, k->err);
-    svgf::Params P;
-    memset(&P, 0, sizeof P);
-    if (e == cudaSuccess) e = apply(k->K, c0, k->c1, B, H, W, 1, P, nullptr, nullptr, s);
-    if (e == cudaSuccess) e = apply(k->K, k->c1, c2, B, H, W, 4, P, nullptr, nullptr, s);
+    if (e == cudaSuccess) e = apply(k->K, c0, k->c1, B, H, W, 1, nullptr, nullptr, nullptr, s);
+    if (e == cudaSuccess) e = apply(k->K, k->c1, c2, B, H, W, 4, T, k->u, k->loss_sum, s);
     return e;
 }
 
@@ -1268,8 +1266,8 @@ cudaError_t kpn_run_grad(svgf_kpn* k, const __nv_bfloat16* feats, const float4* 
     using namespace svgf::kpn;
     cudaError_t e = cudaMemsetAsync(k->grad, 0, sizeof(float) * kParamCount, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(k->loss_sum, 0, sizeof(float), s);
-    if (e == cudaSuccess) e = kpn_run_forward(k, feats, c0, B, H, W, k->c2, s);
-    if (e == cudaSuccess) e = backward_apply(k->K, c0, k->c1, k->c2, T, k->gK, k->u, k->dzA, k->loss_sum, B, H, W, s);
+    if (e == cudaSuccess) e = kpn_run_forward(k, feats, c0, T, B, H, W, k->c2, s);
+    if (e == cudaSuccess) e = backward_apply(k->K, c0, k->c1, k->c2, k->u, k->dzA, B, H, W, s);
     if (e == cudaSuccess) e = wgrad(3, k->x3, k->dzA, k->grad, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess) e = conv(3, true, k->dzA, k->w, k->x3, k->dzB, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess) e = wgrad(2, k->x2, k->dzB, k->grad, B, H, W, k->sm_count, s, k->err);
@@ -1427,7 +1425,7 @@ svgf_status svgf_kpn_load(svgf_kpn* k, const void* host_buf, size_t bytes, void*
 svgf_status svgf_kpn_forward(svgf_kpn* k, const void* feats, const float* c0, int B, int H, int W,
                              float* c2_out, void* stream) {
     if (!kpn_batch_ok(k, feats, c0, B, H, W) || !c2_out || !aligned16(c2_out)) return SVGF_ERR_INVALID_ARG;
-    return kpn_fail(k, kpn_run_forward(k, (const __nv_bfloat16*)feats, (const float4*)c0, B, H, W,
+    return kpn_fail(k, kpn_run_forward(k, (const __nv_bfloat16*)feats, (const float4*)c0, nullptr, B, H, W,
                                        (float4*)c2_out, as_stream(stream)));
 }
 

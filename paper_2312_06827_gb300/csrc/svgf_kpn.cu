@@ -1576,59 +1576,13 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const __grid_constant__
 
 // ---------------------------------------------------------------- softmax + kernel application
 
-// c_out(p) = sum_i K_i(p) c_in(p + d o_i) / sum_{i in image} K_i(p), K planar (K[i][p]).
-// rgb_out: inverse tone map fused, written instead of c_out (channel 3 = var_src.w).
-__global__ void k_apply(const float* __restrict__ K, const float4* __restrict__ c_in, float4* c_out,
-                        int B, int H, int W, int d, Params P, float4* rgb_out,
-                        const float4* __restrict__ var_src) {
-    const long np = (long)B * H * W;
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= W || y >= H) return;
-    {
-        const long base = (long)blockIdx.z * H * W;
-        const long p = base + (long)y * W + x;
-        float s = 0.f, r = 0.f, g = 0.f, b = 0.f;
-#pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
-#pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int qx = x + d * kx, qy = y + d * ky;
-                if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                const float k = __ldg(&K[((ky + 2) * 5 + (kx + 2)) * np + p]);
-                const float4 c = __ldg(&c_in[base + (long)qy * W + qx]);
-                s += k;
-                r = fmaf(k, c.x, r);
-                g = fmaf(k, c.y, g);
-                b = fmaf(k, c.z, b);
-            }
-        const float inv = 1.0f / s;
-        const float4 o = make_float4(r * inv, g * inv, b * inv, 0.f);
-        if (rgb_out) {
-            float3 c = make_float3(o.x, o.y, o.z);
-            if (P.tonemap) {
-                const float l = 0.2126f * c.x + 0.7152f * c.y + 0.0722f * c.z;
-                float f;
-                if (P.inverse_mode == 1) {
-                    f = (1.0f + l) * P.inv_weight;
-                } else {
-                    float dd = 1.0f - P.luma_k * l;
-                    dd = dd < 1e-6f ? 1e-6f : dd;
-                    f = 1.0f / dd;
-                }
-                c = make_float3(c.x * f, c.y * f, c.z * f);
-            }
-            rgb_out[p] = make_float4(c.x, c.y, c.z, var_src ? var_src[p].w : 0.f);
-        } else {
-            c_out[p] = o;
-        }
-    }
-}
+// A kernel application: c_out(p) = sum_i K_i(p) c_in(p + D o_i) / sum_{i in image} K_i(p).  A block
+// of 32 x 8 threads takes 32 x 16 pixels (two a thread) and first copies their colour taps' window
+// (the tile with a margin of 2 D) into shared memory, so that each of the 25 taps is read from
+// there rather than through L1: at dilation 4 the taps reach 8 pixels away and L1 serves few of
+// them.  k_apply_h takes the kernels as FP16, pixel-major (Kh[p][32], the first 25 used; conv
+// EPI 3), k_apply as FP32 planes (K[i][p]; conv EPI 1).
 
-// k_apply with the kernels as FP16, pixel-major (Kh[p][32], the first 25 used; conv EPI 3),
-// the same sums in the same order.  A block of 32 x 8 threads takes 32 x 16 pixels (two a
-// thread) and first copies their colour taps' window (the tile with a margin of 2 D) into shared
-// memory, so that each of the 25 taps is read from there rather than through L1: at dilation 4
-// the taps reach 8 pixels away and L1 serves few of them.
 // The 25 FP16 kernel weights of pixel p (pixel-major, 64 bytes: 25 used) as floats.
 __device__ __forceinline__ void load_kernel_h(const uint4* __restrict__ Kh, long p, float (&kv)[32]) {
 #pragma unroll
@@ -1645,10 +1599,11 @@ __device__ __forceinline__ void load_kernel_h(const uint4* __restrict__ Kh, long
 }
 
 // One kernel application at pixel (x, y), dilation D: the K-weighted mean of the in-image taps
-// (x + D kx, y + D ky), renormalised over them; the colours come from a shared-memory window
-// `win` (pitch `pitch` float4) whose element (wx, wy) is the pixel (x, y).
+// (x + D kx, y + D ky), renormalised over them, and the sum of their weights (w); the colours come
+// from a shared-memory window `win` (pitch `pitch` float4) whose element (wx, wy) is the pixel
+// (x, y).
 template <int D>
-__device__ __forceinline__ float3 apply_taps(const float (&kv)[32], const float4* win, int pitch, int wx, int wy,
+__device__ __forceinline__ float4 apply_taps(const float (&kv)[32], const float4* win, int pitch, int wx, int wy,
                                              int x, int y, int W, int H) {
     float s = 0.f, r = 0.f, g = 0.f, b = 0.f;
 #pragma unroll
@@ -1665,7 +1620,21 @@ __device__ __forceinline__ float3 apply_taps(const float (&kv)[32], const float4
             b = fmaf(k, c.z, b);
         }
     const float inv = 1.0f / s;
-    return make_float3(r * inv, g * inv, b * inv);
+    return make_float4(r * inv, g * inv, b * inv, s);
+}
+
+// The window of a 32 x TYp tile at (x0, y0) with a margin of M pixels, zeros outside the image.
+template <int M, int TYp>
+__device__ __forceinline__ void load_window(float4 (*win)[32 + 2 * M], const float4* __restrict__ img, int x0, int y0,
+                                            int H, int W) {
+    constexpr int HX = 32 + 2 * M, HY = TYp + 2 * M;
+    for (int i = threadIdx.y * 32 + threadIdx.x; i < HX * HY; i += 256) {
+        const int ly = i / HX, lx = i - ly * HX;
+        const int gx = x0 - M + lx, gy = y0 - M + ly;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (gx >= 0 && gx < W && gy >= 0 && gy < H) v = __ldg(&img[(long)gy * W + gx]);
+        win[ly][lx] = v;
+    }
 }
 
 // The inverse tone map of the library's Params (exact or the paper-literal form).
@@ -1693,13 +1662,7 @@ __global__ void __launch_bounds__(256) k_apply_h(const uint4* __restrict__ Kh, c
     __shared__ float4 tile[HY][HX];
     const int x0 = blockIdx.x * TXp, y0 = blockIdx.y * TYp;
     const long base = (long)blockIdx.z * H * W;
-    for (int i = threadIdx.y * 32 + threadIdx.x; i < HX * HY; i += 256) {
-        const int ly = i / HX, lx = i - ly * HX;
-        const int gx = x0 - 2 * D + lx, gy = y0 - 2 * D + ly;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gx >= 0 && gx < W && gy >= 0 && gy < H) v = __ldg(&c_in[base + (long)gy * W + gx]);
-        tile[ly][lx] = v;
-    }
+    load_window<2 * D, TYp>(tile, c_in + base, x0, y0, H, W);
     __syncthreads();
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
@@ -1709,9 +1672,9 @@ __global__ void __launch_bounds__(256) k_apply_h(const uint4* __restrict__ Kh, c
         const long p = base + (long)y * W + x;
         float kv[32];
         load_kernel_h(Kh, p, kv);
-        const float3 o = apply_taps<D>(kv, &tile[0][0], HX, lx + 2 * D, ly + 2 * D, x, y, W, H);
+        const float4 o = apply_taps<D>(kv, &tile[0][0], HX, lx + 2 * D, ly + 2 * D, x, y, W, H);
         if (rgb_out) {
-            const float3 c = inverse_tm(P, o);
+            const float3 c = inverse_tm(P, make_float3(o.x, o.y, o.z));
             rgb_out[p] = make_float4(c.x, c.y, c.z, var_src ? var_src[p].w : 0.f);
         } else {
             c_out[p] = make_float4(o.x, o.y, o.z, 0.f);
@@ -1719,121 +1682,128 @@ __global__ void __launch_bounds__(256) k_apply_h(const uint4* __restrict__ Kh, c
     }
 }
 
-// Backward of the second application and the loss: g2 = 2 (c2 - T) / (3 N); stores
-// gK(p) = sum_c g2 (c1(q_i) - c2) / S2 and u(p) = g2 / S2; accumulates the squared error.
-__global__ void k_bwd_apply2(const float* __restrict__ K, const float4* __restrict__ c1,
-                             const float4* __restrict__ c2, const float4* __restrict__ T, float* gK,
-                             float4* u, float* loss_sum, int B, int H, int W, float scale) {
-    const long np = (long)B * H * W;
-    float sq = 0.f;
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
-    if (x < W && y < H) {
-        const long base = (long)blockIdx.z * H * W;
-        const long p = base + (long)y * W + x;
-        const float4 o = c2[p], t = T[p];
-        const float e0 = o.x - t.x, e1 = o.y - t.y, e2 = o.z - t.z;
-        sq += e0 * e0 + e1 * e1 + e2 * e2;
-        const float g0 = scale * e0, g1 = scale * e1, g2 = scale * e2;
-        float S = 0.f;
-#pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
-#pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int qx = x + 4 * kx, qy = y + 4 * ky;
-                if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                S += K[((ky + 2) * 5 + (kx + 2)) * np + p];
-            }
-        const float rS = 1.0f / S;
-#pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
-#pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int i = (ky + 2) * 5 + (kx + 2);
-                const int qx = x + 4 * kx, qy = y + 4 * ky;
-                float v = 0.f;
-                if (qx >= 0 && qy >= 0 && qx < W && qy < H) {
-                    const float4 q = c1[base + (long)qy * W + qx];
-                    v = (g0 * (q.x - o.x) + g1 * (q.y - o.y) + g2 * (q.z - o.z)) * rS;
-                }
-                gK[i * np + p] = v;
-            }
-        u[p] = make_float4(g0 * rS, g1 * rS, g2 * rS, 0.f);
-    }
-    // block reduction of the squared error (blocks of 32 x 8 threads: one warp per row)
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    __shared__ float red[8];
-    if (threadIdx.x == 0) red[threadIdx.y] = sq;
+// An application of the training forward, kernels as FP32 planes K[i][np].  EPI 0: c_out = the
+// colour, channel 3 zero.  EPI 1: channel 3 = the sum S of the in-image weights (the backward pass
+// divides by it).  EPI 2, the second application of a gradient: c_out as EPI 0, and with the target
+// T the squared error added to *loss_sum and u = g2 / S, g2 = scale (c_out - T) the loss's gradient.
+// A thread's 25 weights are loaded before its taps, so their latency is paid once a pixel, and the
+// taps come from the window: 51 -> 28 us at dilation 1 and 51 -> 38 at dilation 4 with the loss (16
+// crops of 256 x 256; 18 us of that are the weights' bytes).
+template <int D, int EPI>
+__global__ void __launch_bounds__(256, 4) k_apply(const float* __restrict__ K, const float4* __restrict__ c_in,
+                                                  float4* c_out, long np, int H, int W, const float4* __restrict__ T,
+                                                  float4* u, float* loss_sum, float scale) {
+    constexpr int TYp = 16, HX = 32 + 4 * D, HY = TYp + 4 * D;
+    __shared__ float4 tile[HY][HX];
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * TYp;
+    const long base = (long)blockIdx.z * H * W;
+    load_window<2 * D, TYp>(tile, c_in + base, x0, y0, H, W);
     __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += red[w];
-        atomicAdd(loss_sum, s);
+    float sq = 0.f;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        const int lx = threadIdx.x, ly = threadIdx.y + 8 * half;
+        const int x = x0 + lx, y = y0 + ly;
+        if (x >= W || y >= H) continue;
+        const long p = base + (long)y * W + x;
+        float kv[32];
+#pragma unroll
+        for (int i = 0; i < 25; ++i) kv[i] = __ldg(&K[i * np + p]);
+        const float4 o = apply_taps<D>(kv, &tile[0][0], HX, lx + 2 * D, ly + 2 * D, x, y, W, H);
+        c_out[p] = make_float4(o.x, o.y, o.z, EPI == 1 ? o.w : 0.f);
+        if constexpr (EPI == 2) {
+            const float4 t = __ldg(&T[p]);
+            const float e0 = o.x - t.x, e1 = o.y - t.y, e2 = o.z - t.z;
+            sq += e0 * e0 + e1 * e1 + e2 * e2;
+            const float rS = 1.0f / o.w;
+            u[p] = make_float4(scale * e0 * rS, scale * e1 * rS, scale * e2 * rS, 0.f);
+        }
+    }
+    if constexpr (EPI == 2) {
+        // block sum of the squared error, one atomic add a block
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        __shared__ float red[8];
+        if (threadIdx.x == 0) red[threadIdx.y] = sq;
+        __syncthreads();
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
+            float s = 0.f;
+            for (int w = 0; w < 8; ++w) s += red[w];
+            atomicAdd(loss_sum, s);
+        }
     }
 }
 
-// Gradient reaching c1: g1(q) = sum_i [p = q - 4 o_i in image] u(p) K_i(p); then the first
-// application's kernel gradient gK(q) += sum_c g1 (c0(q + o_i) - c1(q)) / S1 and the softmax
-// backward dz_j = K_j (gK_j - sum_i K_i gK_i), written as BF16 [p][32] (zeros past 25).
-__global__ void k_bwd_apply1(const float* __restrict__ K, const float4* __restrict__ u,
-                             const float4* __restrict__ c0, const float4* __restrict__ c1,
-                             const float* __restrict__ gK, __nv_bfloat16* dz, int B, int H, int W) {
-    const long np = (long)B * H * W;
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+// Backward through both applications and the softmax, per pixel q, from u = g2 / S2 and the
+// applications' outputs c1 (channel 3: S1) and c2:
+//   the gradient reaching c1: g1 = sum_i [p = q - 4 o_i in image] u(p) K_i(p);
+//   the kernel's gradient:    gK_i = u (c1(q + 4 o_i) - c2) + g1 (c0(q + o_i) - c1) / S1, each term
+//                             over its in-image taps;
+//   the logits' gradient:     dz_j = K_j (gK_j - sum_i K_i gK_i), BF16 [p][32] (zeros past 25).
+// The second application's term is formed here from shared-memory windows of u, c1 and c0 rather
+// than by a kernel of its own that passes 25 FP32 planes (200 B a pixel written and read back)
+// through memory.  The weights K_j are read again for the last line (from L1) instead of being
+// kept: 25 registers less, four blocks a SM instead of two.  16 crops of 256 x 256: 53 + 188 -> 126
+// us.
+__global__ void __launch_bounds__(256, 4) k_bwd_apply(const float* __restrict__ K, const float4* __restrict__ u,
+                                                      const float4* __restrict__ c0, const float4* __restrict__ c1,
+                                                      const float4* __restrict__ c2, __nv_bfloat16* dz, long np,
+                                                      int H, int W) {
+    __shared__ float4 wu[8 + 16][32 + 16], w1[8 + 16][32 + 16], w0[8 + 4][32 + 4];
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8;
+    const long base = (long)blockIdx.z * H * W;
+    load_window<8, 8>(wu, u + base, x0, y0, H, W);
+    load_window<8, 8>(w1, c1 + base, x0, y0, H, W);
+    load_window<2, 8>(w0, c0 + base, x0, y0, H, W);
+    __syncthreads();
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x >= W || y >= H) return;
-    {
-        const long base = (long)blockIdx.z * H * W;
-        const long q = base + (long)y * W + x;
-        float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+    const int lx = threadIdx.x, ly = threadIdx.y;
+    const long q = base + (long)y * W + x;
+    float g0 = 0.f, g1 = 0.f, g2 = 0.f;
 #pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
+    for (int ky = -2; ky <= 2; ++ky)
 #pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int px = x - 4 * kx, py = y - 4 * ky;
-                if (px < 0 || py < 0 || px >= W || py >= H) continue;
-                const long p = base + (long)py * W + px;
-                const float k = K[((ky + 2) * 5 + (kx + 2)) * np + p];
-                const float4 uu = u[p];
-                g0 = fmaf(k, uu.x, g0);
-                g1 = fmaf(k, uu.y, g1);
-                g2 = fmaf(k, uu.z, g2);
-            }
-        const float4 o = c1[q];
-        float S = 0.f;
-        float Kq[25], gq[25];
-#pragma unroll
-        for (int i = 0; i < 25; ++i) {
-            Kq[i] = K[i * np + q];
-            gq[i] = gK[i * np + q];
+        for (int kx = -2; kx <= 2; ++kx) {
+            const int px = x - 4 * kx, py = y - 4 * ky;
+            if (px < 0 || py < 0 || px >= W || py >= H) continue;
+            const float k = __ldg(&K[((ky + 2) * 5 + (kx + 2)) * np + base + (long)py * W + px]);
+            const float4 uu = wu[ly + 8 - 4 * ky][lx + 8 - 4 * kx];
+            g0 = fmaf(k, uu.x, g0);
+            g1 = fmaf(k, uu.y, g1);
+            g2 = fmaf(k, uu.z, g2);
         }
+    const float4 o1 = w1[ly + 8][lx + 8], o2 = __ldg(&c2[q]), uq = wu[ly + 8][lx + 8];
+    const float rS = 1.0f / o1.w;
+    float gq[25], dot = 0.f;
 #pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
+    for (int ky = -2; ky <= 2; ++ky)
 #pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int qx = x + kx, qy = y + ky;
-                if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                S += Kq[(ky + 2) * 5 + (kx + 2)];
+        for (int kx = -2; kx <= 2; ++kx) {
+            const int i = (ky + 2) * 5 + (kx + 2);
+            float v = 0.f;
+            if (x + 4 * kx >= 0 && y + 4 * ky >= 0 && x + 4 * kx < W && y + 4 * ky < H) {
+                const float4 c = w1[ly + 8 + 4 * ky][lx + 8 + 4 * kx];
+                v = uq.x * (c.x - o2.x) + uq.y * (c.y - o2.y) + uq.z * (c.z - o2.z);
             }
-        const float rS = 1.0f / S;
-#pragma unroll
-        for (int ky = -2; ky <= 2; ++ky)
-#pragma unroll
-            for (int kx = -2; kx <= 2; ++kx) {
-                const int qx = x + kx, qy = y + ky;
-                if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                const float4 c = c0[base + (long)qy * W + qx];
-                gq[(ky + 2) * 5 + (kx + 2)] += (g0 * (c.x - o.x) + g1 * (c.y - o.y) + g2 * (c.z - o.z)) * rS;
+            if (x + kx >= 0 && y + ky >= 0 && x + kx < W && y + ky < H) {
+                const float4 c = w0[ly + 2 + ky][lx + 2 + kx];
+                v += (g0 * (c.x - o1.x) + g1 * (c.y - o1.y) + g2 * (c.z - o1.z)) * rS;
             }
-        float dot = 0.f;
-#pragma unroll
-        for (int i = 0; i < 25; ++i) dot = fmaf(Kq[i], gq[i], dot);
-        unsigned* out = reinterpret_cast<unsigned*>(dz + q * 32);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int a = 2 * i, b = 2 * i + 1;
-            const float va = a < 25 ? Kq[a] * (gq[a] - dot) : 0.f;
-            const float vb = b < 25 ? Kq[b] * (gq[b] - dot) : 0.f;
-            out[i] = pack_bf16(va, vb);
+            gq[i] = v;
+            dot = fmaf(__ldg(&K[i * np + q]), v, dot);
         }
+    uint4* out = reinterpret_cast<uint4*>(dz + q * 32);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        unsigned w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int a = 8 * h + 2 * i, b = a + 1;
+            const float va = a < 25 ? __ldg(&K[(a < 25 ? a : 0) * np + q]) * (gq[a < 25 ? a : 0] - dot) : 0.f;
+            const float vb = b < 25 ? __ldg(&K[(b < 25 ? b : 0) * np + q]) * (gq[b < 25 ? b : 0] - dot) : 0.f;
+            w[i] = pack_bf16(va, vb);
+        }
+        out[h] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -2071,10 +2041,15 @@ cudaError_t wgrad(int layer, const __nv_bfloat16* X, const __nv_bfloat16* dZ, fl
     return layer == 0 ? launch(k_wgrad<16>, 16, WgradCfg<16>::SMEM) : launch(k_wgrad<32>, 32, WgradCfg<32>::SMEM);
 }
 
-cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W,
-                  int dilation, const Params& P, float4* rgb_out, const float4* var_src, cudaStream_t s) {
-    const dim3 grid((W + 31) / 32, (H + 7) / 8, B), block(32, 8);
-    k_apply<<<grid, block, 0, s>>>(K, c_in, c_out, B, H, W, dilation, P, rgb_out, var_src);
+cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W, int dilation,
+                  const float4* T, float4* u, float* loss_sum, cudaStream_t s) {
+    const long np = (long)B * H * W;
+    const float scale = 2.0f / (3.0f * (float)np);
+    const dim3 grid((W + 31) / 32, (H + 15) / 16, B), block(32, 8);
+    if (dilation == 1) k_apply<1, 1><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, nullptr, nullptr, nullptr, 0.f);
+    else if (dilation != 4) return cudaErrorInvalidValue;
+    else if (T) k_apply<4, 2><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, T, u, loss_sum, scale);
+    else k_apply<4, 0><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, nullptr, nullptr, nullptr, 0.f);
     return cudaGetLastError();
 }
 
@@ -2087,16 +2062,10 @@ cudaError_t apply_h(const void* Kh, const float4* c_in, float4* c_out, int B, in
     return cudaGetLastError();
 }
 
-cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2,
-                           const float4* T, float* gK, float4* u, __nv_bfloat16* dz, float* loss_sum,
-                           int B, int H, int W, cudaStream_t s) {
-    const long np = (long)B * H * W;
-    const float scale = 2.0f / (3.0f * (float)np);
+cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2, const float4* u,
+                           __nv_bfloat16* dz, int B, int H, int W, cudaStream_t s) {
     const dim3 grid((W + 31) / 32, (H + 7) / 8, B), block(32, 8);
-    k_bwd_apply2<<<grid, block, 0, s>>>(K, c1, c2, T, gK, u, loss_sum, B, H, W, scale);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_bwd_apply1<<<grid, block, 0, s>>>(K, u, c0, c1, gK, dz, B, H, W);
+    k_bwd_apply<<<grid, block, 0, s>>>(K, u, c0, c1, c2, dz, (long)B * H * W, H, W);
     return cudaGetLastError();
 }
 

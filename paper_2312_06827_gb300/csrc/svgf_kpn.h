@@ -58,16 +58,18 @@ cudaError_t wait_expiry_probe(int tries, int* err, cudaStream_t s);
 // Adds the layer's weight and bias gradients into grad_flat (flat parameter layout).  Waits as in conv.
 cudaError_t wgrad(int layer, const __nv_bfloat16* X, const __nv_bfloat16* dZ, float* grad_flat,
                   int B, int H, int W, int sm_count, cudaStream_t s, int* err);
-// c_out = K-weighted mean of c_in at the given dilation (K planar [25][B*H*W]); with rgb_out, the
-// inverse tone map is fused and rgb_out.w = var_src.w.
-cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W,
-                  int dilation, const Params& P, float4* rgb_out, const float4* var_src, cudaStream_t s);
-// apply with the FP16 pixel-major kernels of conv layer 4.
+// c_out = K-weighted mean of c_in at dilation 1 (channel 3: the sum of the in-image weights) or 4
+// (channel 3 zero), K planar [25][B*H*W].  With a target T (dilation 4) also the squared error, added
+// to *loss_sum, and u = its gradient to c_out over the sum of the in-image weights.
+cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int H, int W, int dilation,
+                  const float4* T, float4* u, float* loss_sum, cudaStream_t s);
+// The same with the FP16 pixel-major kernels of conv layer 4; with rgb_out, the inverse tone map is
+// fused and rgb_out.w = var_src.w.
 cudaError_t apply_h(const void* Kh, const float4* c_in, float4* c_out, int B, int H, int W,
                     int dilation, const Params& P, float4* rgb_out, const float4* var_src, cudaStream_t s);
-cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2,
-                           const float4* T, float* gK, float4* u, __nv_bfloat16* dz, float* loss_sum,
-                           int B, int H, int W, cudaStream_t s);
+// dz [p][32] BF16: the loss's gradient to the logits, from apply's outputs c1, c2 and u.
+cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2, const float4* u,
+                           __nv_bfloat16* dz, int B, int H, int W, cudaStream_t s);
 cudaError_t adam(float* prm, const float* grad, float* m, float* v, float lr, float b1, float b2,
                  float eps, float bc1, float bc2, cudaStream_t s);
 cudaError_t features(int prec, const void* cv, const float4* gbuf, const float* albedo,
