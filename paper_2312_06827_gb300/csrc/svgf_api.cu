@@ -246,8 +246,9 @@ svgf_status run_temporal(svgf_handle* h, const svgf_frame* f, void* cv_out, cuda
 // One a-trous iteration cv_in -> (cv_out | rgb_out with the inverse map fused).
 // need (optional): the pass computes only the 32x32 tiles set in it (need_tx tiles a row); for
 // the separable mode need_h gives the horizontal pass's tiles.
+// chained: another launch of the same call precedes it on the stream.
 svgf_status run_atrous(svgf_handle* h, int iter, const svgf_frame* f, const void* cv_in,
-                       void* cv_out, float4* rgb_out, cudaStream_t s,
+                       void* cv_out, float4* rgb_out, bool chained, cudaStream_t s,
                        const unsigned char* need = nullptr, const unsigned char* need_h = nullptr,
                        int need_tx = 0) {
     const int pr = h->cfg.precision;
@@ -257,16 +258,17 @@ svgf_status run_atrous(svgf_handle* h, int iter, const svgf_frame* f, const void
         {
             LaunchScope L(h, SVGF_K_ATROUS_H, s);
             svgf_status st = L.done(svgf::launch_atrous(pr, h->P, 1, iter, cv_in, (const float4*)f->gbuf_nz,
-                                                        rough, h->sep, nullptr, nullptr, s, need_h, need_tx));
+                                                        rough, h->sep, nullptr, nullptr, chained, s, need_h,
+                                                        need_tx));
             if (st != SVGF_OK) return st;
         }
         LaunchScope L(h, SVGF_K_ATROUS_V, s);
         return L.done(svgf::launch_atrous(pr, h->P, 2, iter, h->sep, (const float4*)f->gbuf_nz, rough,
-                                          cv_out, hist_out, rgb_out, s, need, need_tx));
+                                          cv_out, hist_out, rgb_out, true, s, need, need_tx));
     }
     LaunchScope L(h, SVGF_K_ATROUS_5X5, s);
     return L.done(svgf::launch_atrous(pr, h->P, 0, iter, cv_in, (const float4*)f->gbuf_nz, rough,
-                                      cv_out, hist_out, rgb_out, s, need, need_tx));
+                                      cv_out, hist_out, rgb_out, chained, s, need, need_tx));
 }
 
 svgf_status run_inverse(svgf_handle* h, const void* cv_in, float4* rgb_out, cudaStream_t s) {
@@ -283,7 +285,7 @@ svgf_status run_frame(svgf_handle* h, const svgf_frame* f, float4* rgb_out, cuda
     for (int i = 0; i < n; ++i) {
         const bool last = i == n - 1;
         st = run_atrous(h, i, f, bufs[i & 1], last ? nullptr : bufs[(i + 1) & 1],
-                        last ? rgb_out : nullptr, s);
+                        last ? rgb_out : nullptr, true, s);
         if (st != SVGF_OK) return st;
     }
     return SVGF_OK;
@@ -448,7 +450,7 @@ svgf_status svgf_atrous(svgf_handle* h, int iter, const svgf_frame* f, const flo
         !cv_aligned(h, cv_out))
         return SVGF_ERR_INVALID_ARG;
     if (iter < 0 || iter >= 16) return SVGF_ERR_INVALID_ARG;
-    return run_atrous(h, iter, f, cv_in, cv_out, nullptr, as_stream(stream));
+    return run_atrous(h, iter, f, cv_in, cv_out, nullptr, false, as_stream(stream));
 }
 
 svgf_status svgf_inverse_tonemap(svgf_handle* h, const float* cv_in, float* rgb_out,
@@ -740,12 +742,12 @@ extern "C" svgf_status svgf_atrous_separable_noalloc(svgf_handle* h, int iter,
         LaunchScope L(h, SVGF_K_ATROUS_H, s);
         svgf_status st = L.done(svgf::launch_atrous(h->cfg.precision, h->P, 1, iter, cv_in,
                                                     (const float4*)f->gbuf_nz, rough, scratch,
-                                                    nullptr, nullptr, s));
+                                                    nullptr, nullptr, false, s));
         if (st != SVGF_OK) return st;
     }
     LaunchScope L(h, SVGF_K_ATROUS_V, s);
     return L.done(svgf::launch_atrous(h->cfg.precision, h->P, 2, iter, scratch,
-                                      (const float4*)f->gbuf_nz, rough, cv_out, nullptr, nullptr, s));
+                                      (const float4*)f->gbuf_nz, rough, cv_out, nullptr, nullptr, true, s));
 }
 
 // ---- batched streams --------------------------------------------------------------------------
@@ -1252,10 +1254,10 @@ cudaError_t kpn_run_forward(svgf_kpn* k, const __nv_bfloat16* feats, const float
                             int H, int W, float4* c2, cudaStream_t s) {
     using namespace svgf::kpn;
     cudaError_t e = kpn_zero_err(k, s);
-    if (e == cudaSuccess) e = conv(0, false, feats, k->w, nullptr, k->x1, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(3, false, k->x3, k->w, nullptr, k->K, B, H, W, k->sm_count, s, k->err);
+    if (e == cudaSuccess) e = conv(0, false, feats, k->w, nullptr, k->x1, B, H, W, k->sm_count, false, s, k->err);
+    if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, B, H, W, k->sm_count, true, s, k->err);
+    if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, B, H, W, k->sm_count, true, s, k->err);
+    if (e == cudaSuccess) e = conv(3, false, k->x3, k->w, nullptr, k->K, B, H, W, k->sm_count, true, s, k->err);
     if (e == cudaSuccess) e = apply(k->K, c0, k->c1, B, H, W, 1, nullptr, nullptr, nullptr, s);
     if (e == cudaSuccess) e = apply(k->K, k->c1, c2, B, H, W, 4, T, k->u, k->loss_sum, s);
     return e;
@@ -1269,11 +1271,11 @@ cudaError_t kpn_run_grad(svgf_kpn* k, const __nv_bfloat16* feats, const float4* 
     if (e == cudaSuccess) e = kpn_run_forward(k, feats, c0, T, B, H, W, k->c2, s);
     if (e == cudaSuccess) e = backward_apply(k->K, c0, k->c1, k->c2, k->u, k->dzA, B, H, W, s);
     if (e == cudaSuccess) e = wgrad(3, k->x3, k->dzA, k->grad, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(3, true, k->dzA, k->w, k->x3, k->dzB, B, H, W, k->sm_count, s, k->err);
+    if (e == cudaSuccess) e = conv(3, true, k->dzA, k->w, k->x3, k->dzB, B, H, W, k->sm_count, true, s, k->err);
     if (e == cudaSuccess) e = wgrad(2, k->x2, k->dzB, k->grad, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(2, true, k->dzB, k->w, k->x2, k->dzA, B, H, W, k->sm_count, s, k->err);
+    if (e == cudaSuccess) e = conv(2, true, k->dzB, k->w, k->x2, k->dzA, B, H, W, k->sm_count, true, s, k->err);
     if (e == cudaSuccess) e = wgrad(1, k->x1, k->dzA, k->grad, B, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(1, true, k->dzA, k->w, k->x1, k->dzB, B, H, W, k->sm_count, s, k->err);
+    if (e == cudaSuccess) e = conv(1, true, k->dzA, k->w, k->x1, k->dzB, B, H, W, k->sm_count, true, s, k->err);
     if (e == cudaSuccess) e = wgrad(0, feats, k->dzB, k->grad, B, H, W, k->sm_count, s, k->err);
     if (e == cudaSuccess && loss_out) e = loss_finish(k->loss_sum, loss_out, (long)B * H * W, s);
     return e;
@@ -1356,7 +1358,7 @@ svgf_status svgf_kpn_params_changed(svgf_kpn* k, int reset_adam, void* stream) {
             if (e != cudaSuccess) return kpn_fail(k, e);
         }
     }
-    return kpn_fail(k, svgf::kpn::prep_weights(k->params, k->w, as_stream(stream)));
+    return kpn_fail(k, svgf::kpn::prep_weights(k->params, k->w, false, as_stream(stream)));
 }
 
 // Checkpoint layout (little-endian): magic, version, parameter count, flags (bit 0: Adam state),
@@ -1444,10 +1446,10 @@ svgf_status svgf_kpn_predict(svgf_kpn* k, const void* feats, int B, int H, int W
     } else if (form == 2) {
         if (e == cudaSuccess) e = net_pairs(x, k->w, k->x2, kernels_out, B, H, W, k->sm_count, s, k->err);
     } else {
-        if (e == cudaSuccess) e = conv(0, false, x, k->w, nullptr, k->x1, B, H, W, k->sm_count, s, k->err);
-        if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, B, H, W, k->sm_count, s, k->err);
-        if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, B, H, W, k->sm_count, s, k->err);
-        if (e == cudaSuccess) e = conv(4, false, k->x3, k->w, nullptr, kernels_out, B, H, W, k->sm_count, s, k->err);
+        if (e == cudaSuccess) e = conv(0, false, x, k->w, nullptr, k->x1, B, H, W, k->sm_count, false, s, k->err);
+        if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, B, H, W, k->sm_count, true, s, k->err);
+        if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, B, H, W, k->sm_count, true, s, k->err);
+        if (e == cudaSuccess) e = conv(4, false, k->x3, k->w, nullptr, kernels_out, B, H, W, k->sm_count, true, s, k->err);
     }
     return kpn_fail(k, e);
 }
@@ -1475,7 +1477,7 @@ svgf_status svgf_kpn_train_step(svgf_kpn* k, const void* feats, const float* c0,
     const float bc1 = (float)(1.0 - pow(b1, (double)k->adam_t));
     const float bc2 = (float)(1.0 - pow(b2, (double)k->adam_t));
     e = svgf::kpn::adam(k->params, k->grad, k->adam_m, k->adam_v, lr, (float)b1, (float)b2, 1e-8f, bc1, bc2, s);
-    if (e == cudaSuccess) e = svgf::kpn::prep_weights(k->params, k->w, s);
+    if (e == cudaSuccess) e = svgf::kpn::prep_weights(k->params, k->w, true, s);
     return kpn_fail(k, e);
 }
 
@@ -1485,7 +1487,7 @@ svgf_status svgf_kpn_features(svgf_handle* h, const void* cv, const svgf_frame* 
         !aligned16(feats_out) || !aligned16(f->gbuf_nz) || (c0_out && !aligned16(c0_out)))
         return SVGF_ERR_INVALID_ARG;
     return cuda_fail(h, svgf::kpn::features(h->cfg.precision, cv, (const float4*)f->gbuf_nz, albedo,
-                                            (__nv_bfloat16*)feats_out, (float4*)c0_out, (int)h->n_px,
+                                            (__nv_bfloat16*)feats_out, (float4*)c0_out, (int)h->n_px, false,
                                             as_stream(stream)));
 }
 
@@ -1497,8 +1499,9 @@ svgf_status svgf_kpn_apply(svgf_kpn* k, svgf_handle* h, const void* kernels, con
     using namespace svgf::kpn;
     cudaStream_t s = as_stream(stream);
     const int W = h->cfg.width, H = h->cfg.height;
-    cudaError_t e = apply_h(kernels, (const float4*)c0, k->c1, 1, H, W, 1, h->P, nullptr, nullptr, s);
-    if (e == cudaSuccess) e = apply_h(kernels, k->c1, nullptr, 1, H, W, 4, h->P, (float4*)rgb_out, (const float4*)c0, s);
+    cudaError_t e = apply_h(kernels, (const float4*)c0, k->c1, 1, H, W, 1, h->P, nullptr, nullptr, false, s);
+    if (e == cudaSuccess)
+        e = apply_h(kernels, k->c1, nullptr, 1, H, W, 4, h->P, (float4*)rgb_out, (const float4*)c0, true, s);
     return cuda_fail(h, e);
 }
 
@@ -1514,26 +1517,26 @@ svgf_status svgf_kpn_denoise_frame(svgf_kpn* k, svgf_handle* h, const svgf_frame
     const int W = h->cfg.width, H = h->cfg.height;
     svgf_status st = run_temporal(h, f, h->cv_a, s);
     if (st != SVGF_OK) return st;
-    st = run_atrous(h, 0, f, h->cv_a, h->cv_b, nullptr, s);
+    st = run_atrous(h, 0, f, h->cv_a, h->cv_b, nullptr, true, s);
     if (st != SVGF_OK) return st;
     using namespace svgf::kpn;
     cudaError_t e = kpn_zero_err(k, s);
     if (e == cudaSuccess)
         e = features(h->cfg.precision, h->cv_b, (const float4*)f->gbuf_nz, albedo, k->feats, k->c0,
-                     (int)h->n_px, s);
+                     (int)h->n_px, true, s);
     // inference: the network layer by layer (faster than the four-layer kernel of
     // svgf_kpn_predict's form 0, whose four-slot accumulator rings tie each layer's issue to its
     // own drain every two rows), the kernels as FP16, pixel-major (64 B per pixel instead of 25
     // FP32 planes)
-    if (e == cudaSuccess) e = conv(0, false, k->feats, k->w, nullptr, k->x1, 1, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, 1, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, 1, H, W, k->sm_count, s, k->err);
-    if (e == cudaSuccess) e = conv(4, false, k->x3, k->w, nullptr, k->K, 1, H, W, k->sm_count, s, k->err);
+    if (e == cudaSuccess) e = conv(0, false, k->feats, k->w, nullptr, k->x1, 1, H, W, k->sm_count, true, s, k->err);
+    if (e == cudaSuccess) e = conv(1, false, k->x1, k->w, nullptr, k->x2, 1, H, W, k->sm_count, true, s, k->err);
+    if (e == cudaSuccess) e = conv(2, false, k->x2, k->w, nullptr, k->x3, 1, H, W, k->sm_count, true, s, k->err);
+    if (e == cudaSuccess) e = conv(4, false, k->x3, k->w, nullptr, k->K, 1, H, W, k->sm_count, true, s, k->err);
     // the two applications (one launch computing both, the dilation-1 result recomputed over
     // the reach of the dilation-4 taps in shared memory, measured slower: 152 against 109 us at
     // 1080p)
-    if (e == cudaSuccess) e = apply_h(k->K, k->c0, k->c1, 1, H, W, 1, h->P, nullptr, nullptr, s);
-    if (e == cudaSuccess) e = apply_h(k->K, k->c1, nullptr, 1, H, W, 4, h->P, (float4*)rgb_out, k->c0, s);
+    if (e == cudaSuccess) e = apply_h(k->K, k->c0, k->c1, 1, H, W, 1, h->P, nullptr, nullptr, true, s);
+    if (e == cudaSuccess) e = apply_h(k->K, k->c1, nullptr, 1, H, W, 4, h->P, (float4*)rgb_out, k->c0, true, s);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->launches += 7;   // features, four convolutions, two applications
     if (fallback_tiles) *fallback_tiles = 0;
@@ -1588,7 +1591,7 @@ svgf_status svgf_kpn_denoise_frame(svgf_kpn* k, svgf_handle* h, const svgf_frame
     for (int i = 1; i < n; ++i) {
         const bool last = i == n - 1;
         st = run_atrous(h, i, f, bufs[(i - 1) & 1], last ? nullptr : bufs[i & 1],
-                        last ? k->c2 : nullptr, s, out_m[i], h_m[i], ntx);
+                        last ? k->c2 : nullptr, i > 1, s, out_m[i], h_m[i], ntx);
         if (st != SVGF_OK) return st;
     }
     if (n == 1) {

@@ -39,6 +39,7 @@ template <class S, bool UP>
 __global__ void __launch_bounds__(TILE_X* TILE_Y, kTemporalBlocksPerSM)
 kb_temporal(const __grid_constant__ BatchTemporalArgs A) {
     __shared__ TemporalSmem sm;
+    pdl_wait();
     for (int t = blockIdx.x; t < A.total; t += gridDim.x) {
         const BTemporal& d = A.s[stream_of(A, t)];
         const int lt = t - d.tile_base, by = lt / d.tiles_x, bx = lt - by * d.tiles_x;
@@ -58,6 +59,7 @@ kb_spatial_variance(const __grid_constant__ BatchSpatialArgs A) {
     __shared__ unsigned mask[kThreads / 32];
     __shared__ SpatialSmem sm;
     const int tid = threadIdx.y * TILE_X + threadIdx.x;
+    pdl_wait();
     for (int k0 = 0; (long)k0 * gridDim.x + blockIdx.x < A.total; k0 += kThreads) {
         const long t = (long)(k0 + tid) * gridDim.x + blockIdx.x;
         bool f = false;
@@ -119,17 +121,13 @@ kb_atrous(const __grid_constant__ BatchAtrousArgs A) {
 template <class S>
 cudaError_t temporal(const BatchTemporalArgs& a, int grid, cudaStream_t s) {
     const dim3 block(TILE_X, TILE_Y);
-    if (a.uniform) kb_temporal<S, true><<<grid, block, 0, s>>>(a);
-    else kb_temporal<S, false><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch(false, a.uniform ? kb_temporal<S, true> : kb_temporal<S, false>, grid, block, 0, s, a);
 }
 
 template <class S>
 cudaError_t spatial(const BatchSpatialArgs& a, int grid, cudaStream_t s) {
     const dim3 block(TILE_X, TILE_Y);
-    if (a.uniform) kb_spatial_variance<S, true><<<grid, block, 0, s>>>(a);
-    else kb_spatial_variance<S, false><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch(true, a.uniform ? kb_spatial_variance<S, true> : kb_spatial_variance<S, false>, grid, block, 0, s, a);
 }
 
 // The kernel a launch takes: its form (NSM, UP) follows from the descriptors; `per` from the grid.
@@ -180,8 +178,7 @@ cudaError_t atrous(int mode, int shape, const BatchAtrousArgs& a, int grid, cuda
     int tx, ty;
     atrous_shape(shape, &tx, &ty);
     const auto k = atrous_kernel<S>(mode, shape, atrous_form(a), grid < a.total);
-    k<<<grid, dim3(tx, ty), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch(true, k, grid, dim3(tx, ty), 0, s, a);
 }
 
 template <class S>

@@ -874,6 +874,7 @@ __device__ __forceinline__ void atrous_tile(const Params& P, int W, int H, int i
                                             float4* __restrict__ rgb_out,
                                             const unsigned char* __restrict__ need = nullptr,
                                             int need_tx = 0) {
+    pdl_wait();
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y * ys;
     if (MASK && (x >= W || y >= H || !need[(y >> 5) * need_tx + (x >> 5)])) return;
     const int reach = 2 << (iter + (P.adaptive_start && rough != nullptr ? 1 : 0));

@@ -27,6 +27,7 @@ k_temporal(Params P, const float* __restrict__ noisy, const float4* __restrict__
            int has_history, typename S::Rec* __restrict__ cv_out, typename S::Rec* __restrict__ mom_out,
            typename S::Rec* __restrict__ hist_accum_out, int* __restrict__ tile_flags) {
     __shared__ TemporalSmem sm;
+    pdl_wait();
     temporal_tile<S>(P, P.W, P.H, blockIdx.x * TILE_X, blockIdx.y * TILE_Y,
                      &tile_flags[blockIdx.y * gridDim.x + blockIdx.x], noisy, gbuf, prev_gbuf, mv,
                      hist_prev, mom_prev, has_history, cv_out, mom_out, hist_accum_out, sm);
@@ -45,6 +46,7 @@ k_spatial_variance(Params P, const float4* __restrict__ gbuf, const typename S::
     __shared__ unsigned mask[kThreads / 32];
     __shared__ SpatialSmem sm;
     const int tid = threadIdx.y * TILE_X + threadIdx.x;
+    pdl_wait();
     for (int k0 = 0; (long)k0 * gridDim.x + blockIdx.x < n_tiles; k0 += kThreads) {
         const long t = (long)(k0 + tid) * gridDim.x + blockIdx.x;
         const unsigned b = __ballot_sync(~0u, t < n_tiles && tile_flags[t] != 0);
@@ -188,16 +190,15 @@ cudaError_t launch_temporal(int prec, const Params& P, const float* noisy, const
                             void* hist_accum_out, int* tile_flags, cudaStream_t s) {
     const dim3 grid = tile_grid(P.W, P.H), block(TILE_X, TILE_Y);
 #define SVGF_TEMPORAL(ST)                                                                         \
-    k_temporal<ST><<<grid, block, 0, s>>>(                                                        \
-        P, noisy, gbuf, prev_gbuf, mv, (const ST::Rec*)hist_prev, (const ST::Rec*)mom_prev,       \
+    return launch(                                                                                \
+        false, k_temporal<ST>, grid, block, 0, s, P, noisy, gbuf, prev_gbuf, mv, (const ST::Rec*)hist_prev, (const ST::Rec*)mom_prev,       \
         has_history, (ST::Rec*)cv_out, (ST::Rec*)mom_out, (ST::Rec*)hist_accum_out, tile_flags)
     switch (prec) {
-        case 0: SVGF_TEMPORAL(StoreF32); break;
-        case 1: SVGF_TEMPORAL(Store16<false>); break;
-        default: SVGF_TEMPORAL(Store16<true>); break;
+        case 0: SVGF_TEMPORAL(StoreF32);
+        case 1: SVGF_TEMPORAL(Store16<false>);
+        default: SVGF_TEMPORAL(Store16<true>);
     }
 #undef SVGF_TEMPORAL
-    return cudaGetLastError();
 }
 
 cudaError_t launch_spatial_variance(int prec, const Params& P, const float4* gbuf, const void* mom,
@@ -210,21 +211,21 @@ cudaError_t launch_spatial_variance(int prec, const Params& P, const float4* gbu
     if (e != cudaSuccess) return e;
     const int tiles_x = (int)tiles.x, grid = spatial_grid(n_tiles, sms, &tiles_x, 1);
 #define SVGF_SPATIAL(ST)                                                                        \
-    k_spatial_variance<ST><<<grid, block, 0, s>>>(P, gbuf, (const ST::Rec*)mom, tile_flags, n_tiles, \
-                                                   tiles_x, (ST::Rec*)cv)
+    return launch(true, k_spatial_variance<ST>, grid, block, 0, s, P, gbuf, (const ST::Rec*)mom, tile_flags, \
+                  n_tiles, tiles_x, (ST::Rec*)cv)
     switch (prec) {
-        case 0: SVGF_SPATIAL(StoreF32); break;
-        case 1: SVGF_SPATIAL(Store16<false>); break;
-        default: SVGF_SPATIAL(Store16<true>); break;
+        case 0: SVGF_SPATIAL(StoreF32);
+        case 1: SVGF_SPATIAL(Store16<false>);
+        default: SVGF_SPATIAL(Store16<true>);
     }
 #undef SVGF_SPATIAL
-    return cudaGetLastError();
 }
 
 template <class ST>
-static void atrous_dispatch(int mode, const Params& P, int iter, const void* cv_in,
-                            const float4* gbuf, const float* rough, void* cv_out, void* hist_out,
-                            float4* rgb_out, const unsigned char* need, int need_tx, cudaStream_t s) {
+static cudaError_t atrous_dispatch(int mode, const Params& P, int iter, const void* cv_in,
+                                   const float4* gbuf, const float* rough, void* cv_out, void* hist_out,
+                                   float4* rgb_out, const unsigned char* need, int need_tx, bool chained,
+                                   cudaStream_t s) {
     const int tx = mode == 0 ? SVGF_A5_TX : TILE_X, ty = mode == 0 ? SVGF_A5_TY : TILE_Y;
     const int ys = atrous_row_spacing(mode, iter), rows = ty * ys;
     const dim3 grid((unsigned)((P.W + tx - 1) / tx), (unsigned)(((P.H + rows - 1) / rows) * ys)), block(tx, ty);
@@ -234,33 +235,27 @@ static void atrous_dispatch(int mode, const Params& P, int iter, const void* cv_
     // the 24-tap pass takes the series-only normal term for sharp normal weights
     // (sigma_n >= kSeriesOnlySigma); the two-tap separable passes keep the select form
 #define SVGF_AT(M, NS)                                                                                 \
-    if (need)                                                                                          \
-        k_atrous_need<M, ST, NS><<<grid, block, 0, s>>>(P, iter, in, gbuf, rough, out, hist, rgb_out, need, need_tx); \
-    else                                                                                               \
-        k_atrous<M, ST, NS><<<grid, block, 0, s>>>(P, iter, in, gbuf, rough, out, hist, rgb_out)
+    return need ? launch(chained, k_atrous_need<M, ST, NS>, grid, block, 0, s, P, iter, in, gbuf, rough, out, hist, \
+                         rgb_out, need, need_tx)                                                       \
+                : launch(chained, k_atrous<M, ST, NS>, grid, block, 0, s, P, iter, in, gbuf, rough, out, hist, rgb_out)
     switch (mode) {
         case 0:
-            if (P.sigma_n >= kSeriesOnlySigma) {
-                SVGF_AT(0, true);
-            } else {
-                SVGF_AT(0, false);
-            }
-            break;
-        case 1: SVGF_AT(1, false); break;
-        default: SVGF_AT(2, false); break;
+            if (P.sigma_n >= kSeriesOnlySigma) SVGF_AT(0, true);
+            else SVGF_AT(0, false);
+        case 1: SVGF_AT(1, false);
+        default: SVGF_AT(2, false);
     }
 #undef SVGF_AT
 }
 
 cudaError_t launch_atrous(int prec, const Params& P, int mode, int iter, const void* cv_in,
                           const float4* gbuf, const float* rough, void* cv_out, void* hist_out,
-                          float4* rgb_out, cudaStream_t s, const unsigned char* need, int need_tx) {
+                          float4* rgb_out, bool chained, cudaStream_t s, const unsigned char* need, int need_tx) {
     switch (prec) {
-        case 0: atrous_dispatch<StoreF32>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, s); break;
-        case 1: atrous_dispatch<Store16<false>>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, s); break;
-        default: atrous_dispatch<Store16<true>>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, s); break;
+        case 0: return atrous_dispatch<StoreF32>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, chained, s);
+        case 1: return atrous_dispatch<Store16<false>>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, chained, s);
+        default: return atrous_dispatch<Store16<true>>(mode, P, iter, cv_in, gbuf, rough, cv_out, hist_out, rgb_out, need, need_tx, chained, s);
     }
-    return cudaGetLastError();
 }
 
 static unsigned flat_blocks(long n) {

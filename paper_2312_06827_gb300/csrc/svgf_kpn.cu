@@ -392,6 +392,7 @@ __global__ void __launch_bounds__(128 * NG + 64, 2) k_conv3x3_tc(const __grid_co
         for (unsigned i = 0; i < kSlots; ++i) mbar_init(&drained[i], 128);
         mbar_init(fin);
     }
+    pdl_wait();   // before the tensor memory: the previous launch's blocks may still hold theirs
     if (warp == 0) tmem_alloc(tslot, 32 * kSlots);
     fence_proxy_async();
     fence_before();
@@ -1367,6 +1368,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const __grid_constant__
         }
         mbar_init(fin);
     }
+    pdl_wait();                                      // before the tensor memory, as in k_conv3x3_tc
     if (warp == 0) tmem_alloc(tslot, 128 * kWgSets);
     fence_proxy_async();
     fence_before();
@@ -1660,6 +1662,7 @@ __global__ void __launch_bounds__(256) k_apply_h(const uint4* __restrict__ Kh, c
                                                  const float4* __restrict__ var_src) {
     constexpr int TXp = 32, TYp = 16, HX = TXp + 4 * D, HY = TYp + 4 * D;
     __shared__ float4 tile[HY][HX];
+    pdl_wait();
     const int x0 = blockIdx.x * TXp, y0 = blockIdx.y * TYp;
     const long base = (long)blockIdx.z * H * W;
     load_window<2 * D, TYp>(tile, c_in + base, x0, y0, H, W);
@@ -1695,6 +1698,7 @@ __global__ void __launch_bounds__(256, 4) k_apply(const float* __restrict__ K, c
                                                   float4* u, float* loss_sum, float scale) {
     constexpr int TYp = 16, HX = 32 + 4 * D, HY = TYp + 4 * D;
     __shared__ float4 tile[HY][HX];
+    pdl_wait();
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * TYp;
     const long base = (long)blockIdx.z * H * W;
     load_window<2 * D, TYp>(tile, c_in + base, x0, y0, H, W);
@@ -1749,6 +1753,7 @@ __global__ void __launch_bounds__(256, 4) k_bwd_apply(const float* __restrict__ 
                                                       const float4* __restrict__ c2, __nv_bfloat16* dz, long np,
                                                       int H, int W) {
     __shared__ float4 wu[8 + 16][32 + 16], w1[8 + 16][32 + 16], w0[8 + 4][32 + 4];
+    pdl_wait();
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8;
     const long base = (long)blockIdx.z * H * W;
     load_window<8, 8>(wu, u + base, x0, y0, H, W);
@@ -1814,6 +1819,7 @@ __global__ void __launch_bounds__(256, 4) k_bwd_apply(const float* __restrict__ 
 //  dgrad[l] [9][32][32]:      W_l[co][8 - tap][n = ci] transposed (l >= 1; zero for co >= 25)
 //  bias[l]  [32]
 __global__ void k_prep_weights(const float* __restrict__ prm, WeightPtrs w) {
+    pdl_wait();
     const int l = blockIdx.y;
     const int cin = cin_of(l), cout = cout_of(l), cip = cin_pad_of(l);
     const float* Wl = prm + param_offset(l);
@@ -1834,6 +1840,7 @@ __global__ void k_prep_weights(const float* __restrict__ prm, WeightPtrs w) {
 
 __global__ void k_adam(float* prm, const float* __restrict__ grad, float* m, float* v, int n,
                        float lr, float b1, float b2, float eps, float bc1, float bc2) {
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float g = grad[i];
         const float mi = b1 * m[i] + (1.0f - b1) * g;
@@ -1850,6 +1857,7 @@ template <class S>
 __global__ void k_features_t(const typename S::Rec* __restrict__ cv, const float4* __restrict__ gbuf,
                              const float* __restrict__ albedo, __nv_bfloat16* feat, float4* c0,
                              int npx) {
+    pdl_wait();
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npx; p += gridDim.x * blockDim.x) {
         const float4 c = S::ld_cv(cv, p);
         const float4 g = gbuf[p];
@@ -1878,9 +1886,8 @@ unsigned flat_grid(long n, int threads) {
 
 }  // namespace
 
-cudaError_t prep_weights(const float* prm, const WeightPtrs& w, cudaStream_t s) {
-    k_prep_weights<<<dim3(36, 4), 256, 0, s>>>(prm, w);
-    return cudaGetLastError();
+cudaError_t prep_weights(const float* prm, const WeightPtrs& w, bool chained, cudaStream_t s) {
+    return launch(chained, k_prep_weights, dim3(36, 4), 256, 0, s, prm, w);
 }
 
 namespace {
@@ -1938,7 +1945,7 @@ static cudaError_t encode_rows(CUtensorMap* map, const __nv_bfloat16* in, int CI
 }
 
 cudaError_t conv(int layer, bool dgrad, const __nv_bfloat16* in, const WeightPtrs& w,
-                 const __nv_bfloat16* mask, void* out, int B, int H, int W, int sm_count,
+                 const __nv_bfloat16* mask, void* out, int B, int H, int W, int sm_count, bool chained,
                  cudaStream_t s, int* err) {
     {
         const int chunk = conv_chunk(B, H, W, sm_count);
@@ -1956,8 +1963,8 @@ cudaError_t conv(int layer, bool dgrad, const __nv_bfloat16* in, const WeightPtr
             CUtensorMap rows;
             e = encode_rows(&rows, in, ci, B, H, W);
             if (e != cudaSuccess) return e;
-            kernel<<<grid, 128 * ng + 64, smem, s>>>(rows, in, wt, bias, mask, out, B, H, W, chunk, err);
-            return cudaGetLastError();
+            return svgf::launch(chained, kernel, grid, 128 * ng + 64, smem, s, rows, in, wt, bias, mask, out, B, H, W,
+                                chunk, err);
         };
         if (!dgrad) {
             if (layer == 0) return launch(k_conv3x3_tc<16, 0, 2>, 16, 2, w.fwd[0], w.bias[0]);
@@ -2035,8 +2042,8 @@ cudaError_t wgrad(int layer, const __nv_bfloat16* X, const __nv_bfloat16* dZ, fl
         if (e == cudaSuccess) e = encode_rows(&dmap, dZ, 32, B, H, W, tc::M);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kWgThreads, smem, s>>>(xmap, dmap, dW, db, B, H, W, chunk, cin_of(layer), cout_of(layer), err);
-        return cudaGetLastError();
+        return svgf::launch(true, kernel, grid, kWgThreads, smem, s, xmap, dmap, dW, db, B, H, W, chunk, cin_of(layer),
+                            cout_of(layer), err);
     };
     return layer == 0 ? launch(k_wgrad<16>, 16, WgradCfg<16>::SMEM) : launch(k_wgrad<32>, 32, WgradCfg<32>::SMEM);
 }
@@ -2046,44 +2053,39 @@ cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int 
     const long np = (long)B * H * W;
     const float scale = 2.0f / (3.0f * (float)np);
     const dim3 grid((W + 31) / 32, (H + 15) / 16, B), block(32, 8);
-    if (dilation == 1) k_apply<1, 1><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, nullptr, nullptr, nullptr, 0.f);
-    else if (dilation != 4) return cudaErrorInvalidValue;
-    else if (T) k_apply<4, 2><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, T, u, loss_sum, scale);
-    else k_apply<4, 0><<<grid, block, 0, s>>>(K, c_in, c_out, np, H, W, nullptr, nullptr, nullptr, 0.f);
-    return cudaGetLastError();
+    if (dilation != 1 && dilation != 4) return cudaErrorInvalidValue;
+    return launch(true, dilation == 1 ? k_apply<1, 1> : T ? k_apply<4, 2> : k_apply<4, 0>, grid, block, 0, s, K, c_in,
+                  c_out, np, H, W, T, u, loss_sum, scale);
 }
 
 cudaError_t apply_h(const void* Kh, const float4* c_in, float4* c_out, int B, int H, int W,
-                    int dilation, const Params& P, float4* rgb_out, const float4* var_src, cudaStream_t s) {
+                    int dilation, const Params& P, float4* rgb_out, const float4* var_src, bool chained, cudaStream_t s) {
     const dim3 grid((W + 31) / 32, (H + 15) / 16, B), block(32, 8);
-    if (dilation == 1) k_apply_h<1><<<grid, block, 0, s>>>((const uint4*)Kh, c_in, c_out, H, W, P, rgb_out, var_src);
-    else if (dilation == 4) k_apply_h<4><<<grid, block, 0, s>>>((const uint4*)Kh, c_in, c_out, H, W, P, rgb_out, var_src);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    if (dilation != 1 && dilation != 4) return cudaErrorInvalidValue;
+    return launch(chained, dilation == 1 ? k_apply_h<1> : k_apply_h<4>, grid, block, 0, s, (const uint4*)Kh, c_in, c_out,
+                  H, W, P, rgb_out, var_src);
 }
 
 cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2, const float4* u,
                            __nv_bfloat16* dz, int B, int H, int W, cudaStream_t s) {
     const dim3 grid((W + 31) / 32, (H + 7) / 8, B), block(32, 8);
-    k_bwd_apply<<<grid, block, 0, s>>>(K, u, c0, c1, c2, dz, (long)B * H * W, H, W);
-    return cudaGetLastError();
+    return launch(true, k_bwd_apply, grid, block, 0, s, K, u, c0, c1, c2, dz, (long)B * H * W, H, W);
 }
 
 cudaError_t adam(float* prm, const float* grad, float* m, float* v, float lr, float b1, float b2,
                  float eps, float bc1, float bc2, cudaStream_t s) {
-    k_adam<<<flat_grid(kParamCount, 256), 256, 0, s>>>(prm, grad, m, v, kParamCount, lr, b1, b2, eps, bc1, bc2);
-    return cudaGetLastError();
+    return launch(true, k_adam, flat_grid(kParamCount, 256), 256, 0, s, prm, grad, m, v, kParamCount, lr, b1, b2, eps,
+                  bc1, bc2);
 }
 
 cudaError_t features(int prec, const void* cv, const float4* gbuf, const float* albedo,
-                     __nv_bfloat16* feat, float4* c0, int npx, cudaStream_t s) {
+                     __nv_bfloat16* feat, float4* c0, int npx, bool chained, cudaStream_t s) {
     const unsigned g = flat_grid(npx, 256);
     switch (prec) {
-        case 0: k_features_t<dev::StoreF32><<<g, 256, 0, s>>>((const float4*)cv, gbuf, albedo, feat, c0, npx); break;
-        case 1: k_features_t<dev::Store16<false>><<<g, 256, 0, s>>>((const uint2*)cv, gbuf, albedo, feat, c0, npx); break;
-        default: k_features_t<dev::Store16<true>><<<g, 256, 0, s>>>((const uint2*)cv, gbuf, albedo, feat, c0, npx); break;
+        case 0: return launch(chained, k_features_t<dev::StoreF32>, g, 256, 0, s, (const float4*)cv, gbuf, albedo, feat, c0, npx);
+        case 1: return launch(chained, k_features_t<dev::Store16<false>>, g, 256, 0, s, (const uint2*)cv, gbuf, albedo, feat, c0, npx);
+        default: return launch(chained, k_features_t<dev::Store16<true>>, g, 256, 0, s, (const uint2*)cv, gbuf, albedo, feat, c0, npx);
     }
-    return cudaGetLastError();
 }
 
 namespace {
@@ -2171,6 +2173,7 @@ __global__ void k_tile_select(const float4* __restrict__ plain, const unsigned c
 }
 
 __global__ void k_loss_finish(const float* sum, float* loss_out, float inv_n) {
+    pdl_wait();
     if (threadIdx.x == 0) *loss_out = *sum * inv_n;
 }
 }  // namespace
@@ -2195,8 +2198,7 @@ cudaError_t tile_select(const float4* plain, const unsigned char* flags, float4*
 }
 
 cudaError_t loss_finish(const float* sum, float* loss_out, long n, cudaStream_t s) {
-    k_loss_finish<<<1, 32, 0, s>>>(sum, loss_out, 1.0f / (3.0f * (float)n));
-    return cudaGetLastError();
+    return launch(true, k_loss_finish, 1, 32, 0, s, sum, loss_out, 1.0f / (3.0f * (float)n));
 }
 
 }  // namespace kpn

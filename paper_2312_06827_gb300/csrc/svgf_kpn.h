@@ -31,7 +31,9 @@ struct WeightPtrs {
     float* bias[4];            // [32]
 };
 
-cudaError_t prep_weights(const float* prm, const WeightPtrs& w, cudaStream_t s);
+// The launchers below take `chained` as launch() does; those without it follow another launch of
+// the same call and are chained.
+cudaError_t prep_weights(const float* prm, const WeightPtrs& w, bool chained, cudaStream_t s);
 // dgrad = false: layer forward (layers 0..2: + bias, ReLU, BF16; layer 3: + bias and the softmax,
 // the kernels K as 25 FP32 planes [25][B*H*W]).  dgrad = true: data gradient of layer `layer` (1..3) masked by
 // (mask > 0), BF16.
@@ -39,7 +41,7 @@ cudaError_t prep_weights(const float* prm, const WeightPtrs& w, cudaStream_t s);
 // used; read by apply_h).
 // On the tcgen05 tensor cores; a wait that gives up sets kErrWaitGaveUp in *err (a device int).
 cudaError_t conv(int layer, bool dgrad, const __nv_bfloat16* in, const WeightPtrs& w,
-                 const __nv_bfloat16* mask, void* out, int B, int H, int W, int sm_count,
+                 const __nv_bfloat16* mask, void* out, int B, int H, int W, int sm_count, bool chained,
                  cudaStream_t s, int* err);
 // The four layers in one tcgen05 kernel: features [B][H][W][16] in, the softmax weights out as
 // conv layer 4 writes them (FP16, pixel-major, 64 B per pixel), bit for bit; the activations
@@ -66,14 +68,14 @@ cudaError_t apply(const float* K, const float4* c_in, float4* c_out, int B, int 
 // The same with the FP16 pixel-major kernels of conv layer 4; with rgb_out, the inverse tone map is
 // fused and rgb_out.w = var_src.w.
 cudaError_t apply_h(const void* Kh, const float4* c_in, float4* c_out, int B, int H, int W,
-                    int dilation, const Params& P, float4* rgb_out, const float4* var_src, cudaStream_t s);
+                    int dilation, const Params& P, float4* rgb_out, const float4* var_src, bool chained, cudaStream_t s);
 // dz [p][32] BF16: the loss's gradient to the logits, from apply's outputs c1, c2 and u.
 cudaError_t backward_apply(const float* K, const float4* c0, const float4* c1, const float4* c2, const float4* u,
                            __nv_bfloat16* dz, int B, int H, int W, cudaStream_t s);
 cudaError_t adam(float* prm, const float* grad, float* m, float* v, float lr, float b1, float b2,
                  float eps, float bc1, float bc2, cudaStream_t s);
 cudaError_t features(int prec, const void* cv, const float4* gbuf, const float* albedo,
-                     __nv_bfloat16* feat, float4* c0, int npx, cudaStream_t s);
+                     __nv_bfloat16* feat, float4* c0, int npx, bool chained, cudaStream_t s);
 // Fallback: per 32x32 tile, flag = (standard deviation of the luminance of c0.xyz over the tile
 // > thr), counted into *count.
 cudaError_t tile_flags(const float4* c0, int H, int W, float thr, unsigned char* flags, int* count,
