@@ -1745,10 +1745,11 @@ __global__ void __launch_bounds__(256, 4) k_apply(const float* __restrict__ K, c
 //   the logits' gradient:     dz_j = K_j (gK_j - sum_i K_i gK_i), BF16 [p][32] (zeros past 25).
 // The second application's term is formed here from shared-memory windows of u, c1 and c0 rather
 // than by a kernel of its own that passes 25 FP32 planes (200 B a pixel written and read back)
-// through memory.  The weights K_j are read again for the last line (from L1) instead of being
-// kept: 25 registers less, four blocks a SM instead of two.  16 crops of 256 x 256: 53 + 188 -> 126
-// us.
-__global__ void __launch_bounds__(256, 4) k_bwd_apply(const float* __restrict__ K, const float4* __restrict__ u,
+// through memory.  Bound by the latency of its weight loads: the weights K_j are read again for the
+// last line (from L1) instead of being kept, and the budget is five blocks a SM (48 registers):
+// 566 us a training step of 16 crops of 256 x 256, against 579, 598 and 644 with four, three and
+// two blocks.  The two kernels before took 53 + 188 us of that step, this one about 115.
+__global__ void __launch_bounds__(256, 5) k_bwd_apply(const float* __restrict__ K, const float4* __restrict__ u,
                                                       const float4* __restrict__ c0, const float4* __restrict__ c1,
                                                       const float4* __restrict__ c2, __nv_bfloat16* dz, long np,
                                                       int H, int W) {
