@@ -59,7 +59,9 @@ cudaError_t launch(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, si
     c.stream = s;
     c.attrs = at;
     c.numAttrs = chained ? 1 : 0;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // reported here, not left for the thread's next check
+    return e;
 }
 #endif
 
