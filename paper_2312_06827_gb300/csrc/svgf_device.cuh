@@ -649,7 +649,8 @@ __device__ __forceinline__ void spatial_variance_tile_r(const Params& P, int W, 
                     r2 = fmaf(w[a] * d, d, r2);
                 }
                 const float t = sw + rw, d = row_mean - mean, f = __fdiv_rn(rw, t);
-                m2 += fmaf(__fmul_rn(d, d), __fmul_rn(sw, f), r2);
+                // (sw f d) d: 0 on the first row, where d is a luminance whose square may overflow
+                m2 += fmaf(__fmul_rn(__fmul_rn(sw, f), d), d, r2);
                 mean = fmaf(d, f, mean);
                 sw = t;
             }

@@ -65,3 +65,24 @@ def test_weights_around_the_series_switch(w, h, spread, sigma_n):
     # the stage's bar: 1e-5 of the value, and the rounding that FP32 luminances carry
     tol = VAR_TOL * ref + 8 * U * l.max() * np.sqrt(ref)
     assert np.all(np.abs(got - ref) <= tol), np.abs(got - ref).max()
+
+
+@pytest.mark.parametrize("radius", [2, 3])
+def test_large_luminances_without_tone_map(radius):
+    """Linear radiances whose square is past FP32's range but whose variance is not: the estimate is
+    formed from deviations and stays finite."""
+    w, h = 35, 10
+    rng = np.random.default_rng(radius)
+    gbuf = np.zeros((h, w, 4), np.float32)
+    gbuf[..., 2], gbuf[..., 3] = 1.0, 5.0
+    noisy = (3e19 * (1.0 + 1e-3 * rng.standard_normal((h, w, 3)))).astype(np.float32)
+    cfg = svgf.default_config(w, h)
+    cfg.tonemap, cfg.spatial_var_radius = 0, radius
+    d = svgf.Denoiser(cfg)
+    cv = torch.empty(h, w, 4, device="cuda")
+    d.reproject_accumulate(svgf.make_frame(dev(noisy), dev(gbuf), dev(np.zeros((h, w, 2))), dev(np.full((h, w), 0.5))), cv)
+    got = cv[..., 3].cpu().numpy().astype(np.float64)
+    l = noisy.astype(np.float64) @ LUMA
+    ref = first_frame_variance(l, gbuf.astype(np.float64), cfg.sigma_z, cfg.sigma_n, float(np.float32(cfg.eps)), radius)
+    tol = VAR_TOL * ref + 8 * U * l.max() * np.sqrt(ref)
+    assert np.all(np.abs(got - ref) <= tol), np.abs(got / ref - 1).max()
