@@ -39,3 +39,12 @@ def test_gradients_at_tile_edges(B, H, W):
             # the bar of the per-layer gradient tests: 1 % of the norm (BF16 rounding boundaries that
             # FP32 and FP64 sums fall on either side of)
             assert np.linalg.norm(g - o) <= 0.01 * np.linalg.norm(o), (ci, co, n)
+
+
+@pytest.mark.parametrize("B,H,W", [(700, 2, 20), (330, 9, 40), (110, 2, 300), (1300, 1, 17)])
+def test_gradients_of_more_chunks_than_blocks(B, H, W):
+    """More 128-pixel columns than the grid's blocks, so that the blocks take several chunks one after
+    the other and carry their rings' slots and phases from one to the next."""
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert B * -(-W // 128) > blocks                     # a chunk is then a whole column
+    test_gradients_at_tile_edges(B, H, W)
