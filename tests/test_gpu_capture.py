@@ -85,3 +85,63 @@ def test_two_streams_interleaved_equal_one_after_the_other():
     for i in range(2):
         for t in range(4):
             assert torch.equal(want[i][t], got[i][t]), (i, t)
+
+
+@pytest.mark.parametrize("fresh", [True, False])
+def test_captured_learned_frame_equals_direct_frame(fresh):
+    """The longest chain: ten launches, and on a handle's first use a memset between two of them."""
+    w, h = 333, 140
+    frames = frames_of(w, h, 2)
+    albedo = torch.from_numpy(np.random.default_rng(3).random((h, w, 3)).astype(np.float32)).cuda()
+    outs = []
+    for captured in (False, True):
+        d, k = svgf.Denoiser(svgf.default_config(w, h)), svgf.KPN(w * h, train=False)
+        k.init_params(seed=4, last_scale=1.0)
+        o = torch.zeros(h, w, 4, device="cuda")
+        if fresh:
+            d.denoise_frame(frames[0], o)
+        else:
+            k.denoise_frame(d, frames[0], albedo, o)
+        torch.cuda.synchronize()
+        o.zero_()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+                k.denoise_frame(d, frames[1], albedo, o)
+            g.replay()
+        else:
+            k.denoise_frame(d, frames[1], albedo, o)
+        torch.cuda.synchronize()
+        assert k.check_device() == 0
+        outs.append(o)
+    assert float(outs[0][..., :3].abs().max()) > 0
+    assert torch.equal(*outs)
+
+
+@pytest.mark.parametrize("fresh", [True, False])
+def test_captured_training_step_equals_direct_step(fresh):
+    """One block adds up each sum here, so that the order of its additions is the same on every run."""
+    B, H, W = 1, 1, 30
+    rng = np.random.default_rng(7)
+    feats = torch.from_numpy(rng.standard_normal((B, H, W, 16)).astype(np.float32)).cuda().bfloat16().view(torch.int16)
+    c0, target = (torch.from_numpy(rng.random((B, H, W, 4)).astype(np.float32)).cuda() for _ in range(2))
+    got = []
+    for captured in (False, True):
+        k = svgf.KPN(B * H * W)
+        k.init_params(seed=1, last_scale=1.0)
+        if not fresh:
+            k.train_step(feats, c0, target)
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+                loss = k.train_step(feats, c0, target)
+            g.replay()
+        else:
+            loss = k.train_step(feats, c0, target)
+        torch.cuda.synchronize()
+        assert k.check_device() == 0
+        got.append([x.clone() for x in (loss, k.grad, k.params, k.adam_m, k.adam_v)])
+    assert float(got[0][1].abs().max()) > 0
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
