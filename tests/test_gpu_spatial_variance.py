@@ -86,3 +86,32 @@ def test_large_luminances_without_tone_map(radius):
     ref = first_frame_variance(l, gbuf.astype(np.float64), cfg.sigma_z, cfg.sigma_n, float(np.float32(cfg.eps)), radius)
     tol = VAR_TOL * ref + 8 * U * l.max() * np.sqrt(ref)
     assert np.all(np.abs(got - ref) <= tol), np.abs(got / ref - 1).max()
+
+
+def first_frame(noisy, gbuf, cfg):
+    """The temporal stage's colour + variance and the luminances it estimated the variance from."""
+    h, w = gbuf.shape[:2]
+    d = svgf.Denoiser(cfg)
+    cv, hist, mom = (torch.empty(h, w, 4, device="cuda") for _ in range(3))
+    d.reproject_accumulate(svgf.make_frame(dev(noisy), dev(gbuf), dev(np.zeros((h, w, 2))), dev(np.full((h, w), 0.5))), cv)
+    d.history_export(hist, mom)
+    return cv[..., 3].cpu().numpy().astype(np.float64), mom[..., 0].cpu().numpy().astype(np.float64)
+
+
+def test_small_noise_on_a_large_mean():
+    """Noise of 0.1 % of the luminance: the estimate's rounding is of the size of the deviations, not of
+    the luminance.  Against the definition in FP64 from the FP32 luminances themselves.
+
+    The bar, u = 2^-24: depth is constant and |e| < 1, so a weight is off by at most 40 u (the bound
+    of one tap), which moves a weighted variance by at most twice that; the deviations, sums, quotients
+    and merges 48 u."""
+    w, h = 90, 40
+    rng = np.random.default_rng(11)
+    n = np.array([0.0, 0.0, 1.0]) + 0.1 * rng.standard_normal((h, w, 3))
+    n /= np.linalg.norm(n, axis=-1, keepdims=True)
+    gbuf = np.concatenate([n, np.full((h, w, 1), 5.0)], -1).astype(np.float32)
+    cfg = svgf.default_config(w, h)
+    cfg.sigma_n = 2.0
+    got, l = first_frame(0.7 * (1.0 + 1e-3 * rng.standard_normal((h, w, 3))), gbuf, cfg)
+    ref = first_frame_variance(l, gbuf.astype(np.float64), cfg.sigma_z, cfg.sigma_n, float(np.float32(cfg.eps)))
+    assert np.all(np.abs(got - ref) <= 128 * U * ref), np.abs(got / ref - 1.0).max() / U
