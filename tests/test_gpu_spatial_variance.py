@@ -115,3 +115,51 @@ def test_small_noise_on_a_large_mean():
     got, l = first_frame(0.7 * (1.0 + 1e-3 * rng.standard_normal((h, w, 3))), gbuf, cfg)
     ref = first_frame_variance(l, gbuf.astype(np.float64), cfg.sigma_z, cfg.sigma_n, float(np.float32(cfg.eps)))
     assert np.all(np.abs(got - ref) <= 128 * U * ref), np.abs(got / ref - 1.0).max() / U
+
+
+@pytest.mark.parametrize("radius", [1, 3, 7])
+@pytest.mark.parametrize("sigma_n,what", [(1.0, "depth"), (1.0, "normal"), (128.0, "normal")])
+def test_one_tap_weight_against_fp64(radius, sigma_n, what):
+    """The weight w of a single tap, read off the variance of two samples 0 and m, w m^2 / (1 + w)^2:
+    pairs of pixels of one row, so far apart (opposed normals between them) that nothing else has
+    weight.  `depth` sweeps exp(e) over e = 0 .. -85, `normal` (1 - t)^sigma_n through t = 0 .. 1/32,
+    where log(1 - t) is a series, and on to 0.2.
+
+    The bar, u = 2^-24, to first order.  Of w: exp 6 u (ex2.approx 4 u, the correction 2 u); an
+    exponent e that is off by some k u |e| moves w by k u |e|: the FP32 depth or t 4 u, the
+    logarithm 3 u, their product 1 u.  Of the variance from w: the two sums and the mean 2 u each, the
+    deviation twice, the products, the merge of the rows and the final quotients 12 u.  In all
+    8 u |e| + 24 u; taken as 8 u |e| + 32 u.
+
+    Roundings have no sign, and the exponential unit's bias (-0.85 u over most of `depth`'s range) is put
+    back by half a unit: that leaves 0.35 u, and the mean of 500 roundings of 1 u rms another 0.05 u, of
+    which five are allowed: 0.6 u."""
+    n, step = 500, 2 + radius
+    w = n * step
+    s = np.linspace(0.0, 1.0, n)
+    gbuf = np.zeros((1, w, 4), np.float32)
+    gbuf[..., 2] = -1.0                                    # between the pairs
+    a, b = np.arange(n) * step, np.arange(n) * step + 1
+    gbuf[0, a, 2] = 1.0
+    if what == "depth":
+        gbuf[0, b, 2] = 1.0
+        gbuf[0, b, 3] = 85.0 * s                          # eps = 1, sigma_z = 0: e = -|dz|
+    else:
+        t = np.where(s < 0.8, s / 0.8 / 32.0, 1 / 32.0 + (s - 0.8) / 0.2 * (0.2 - 1 / 32.0))
+        gbuf[0, b, 0], gbuf[0, b, 2] = np.sqrt(t * (2.0 - t)), 1.0 - t
+    noisy = np.zeros((1, w, 3), np.float32)
+    noisy[0, b] = 1.0
+    cfg = svgf.default_config(w, 1)
+    cfg.tonemap, cfg.spatial_var_radius = 0, radius
+    cfg.sigma_z, cfg.sigma_n, cfg.eps = 0.0, sigma_n, 1.0
+    got, l = (x[0] for x in first_frame(noisy, gbuf, cfg))
+    g = gbuf[0].astype(np.float64)
+    t = 0.5 * ((g[a, :3] - g[b, :3]) ** 2).sum(-1)
+    e = sigma_n * np.log1p(-t) - np.abs(g[a, 3] - g[b, 3])
+    wt = np.exp(e)
+    ref = wt * l[b] ** 2 / (1.0 + wt) ** 2
+    for p in (a, b):
+        rel = np.abs(got[p] / ref - 1.0)
+        assert np.all(rel <= U * (8.0 * np.abs(e) + 32.0)), (rel / U / (8.0 * np.abs(e) + 32.0)).max()
+        if what == "depth":
+            assert abs(np.mean(got[p] / ref - 1.0)) <= 0.6 * U
