@@ -35,16 +35,8 @@ __device__ __forceinline__ int stream_of(const A& a, int t) {
     return lo;
 }
 
-// Resident blocks per SM of the temporal kernel: the single-frame kernel's four, but three for FP32
-// storage with per-stream parameters, whose registers spilled 152 bytes a thread at four (60 at
-// three).  Eight streams of 640x360 to 2560x1440 (13.8 Mpixel), at three / four blocks: FP32
-// per-stream 479 / 514 us, FP32 launch-wide 461 / 457, 16-bit per-stream 447 / 428, 16-bit
-// launch-wide 427 / 379.
 template <class S, bool UP>
-constexpr int kBatchTemporalBlocksPerSM = !UP && sizeof(typename S::Rec) == 16 ? 3 : kTemporalBlocksPerSM;
-
-template <class S, bool UP>
-__global__ void __launch_bounds__(TILE_X* TILE_Y, (kBatchTemporalBlocksPerSM<S, UP>))
+__global__ void __launch_bounds__(TILE_X* TILE_Y, kTemporalBlocksPerSM)
 kb_temporal(const __grid_constant__ BatchTemporalArgs A) {
     __shared__ TemporalSmem sm;
     pdl_wait();
