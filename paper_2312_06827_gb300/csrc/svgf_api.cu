@@ -759,7 +759,6 @@ struct svgf_batch {
     int sm_count = 0;
     int atrous_shape = 0;     // tile shape index of the batched a-trous kernel
     int atrous_bps = 0;       // a-trous grid: blocks per SM of the persistent grid, 0 = one per tile
-    int stage_bps = 0;        // temporal / spatial-variance grid, same convention
     int use_graph = 0;
     cudaGraphExec_t exec = nullptr;
     char last_error[256] = {0};
@@ -786,7 +785,7 @@ svgf_status batch_fail(svgf_batch* b, cudaError_t e) {
     return SVGF_ERR_CUDA;
 }
 
-// Grid of a batched launch: bps blocks per SM walking the tiles with a grid stride, or, for
+// Grid of a batched a-trous launch: bps blocks per SM walking the tiles with a grid stride, or, for
 // bps = 0, one block per tile (the hardware block scheduler then balances uneven tiles).
 int grid_for(int total, int sm_count, int bps) {
     if (bps <= 0) return total;
@@ -847,8 +846,7 @@ svgf_status batch_temporal(svgf_batch* b, int i0, int i1, const svgf_frame* fram
     ta.P = sa.P = h0->P;
     {
         LaunchScope L(h0, SVGF_K_TEMPORAL, s);
-        svgf_status st = L.done(svgf::launch_batch_temporal(b->cfg.precision, ta,
-                                                            grid_for(total, b->sm_count, b->stage_bps), s));
+        svgf_status st = L.done(svgf::launch_batch_temporal(b->cfg.precision, ta, s));
         if (st != SVGF_OK) return st;
     }
     {

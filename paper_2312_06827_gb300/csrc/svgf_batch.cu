@@ -7,9 +7,9 @@
 
 namespace svgf {
 
-cudaError_t launch_batch_temporal_f32(const BatchTemporalArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_batch_temporal_f16(const BatchTemporalArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_batch_temporal_bf16(const BatchTemporalArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_batch_temporal_f32(const BatchTemporalArgs& a, cudaStream_t s);
+cudaError_t launch_batch_temporal_f16(const BatchTemporalArgs& a, cudaStream_t s);
+cudaError_t launch_batch_temporal_bf16(const BatchTemporalArgs& a, cudaStream_t s);
 cudaError_t launch_batch_spatial_f32(const BatchSpatialArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_batch_spatial_f16(const BatchSpatialArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_batch_spatial_bf16(const BatchSpatialArgs& a, int grid, cudaStream_t s);
@@ -28,11 +28,11 @@ bool same_params_but_size(const Params& a, const Params& b) {
     return memcmp(&x, &y, sizeof(Params)) == 0;
 }
 
-cudaError_t launch_batch_temporal(int prec, const BatchTemporalArgs& a, int grid, cudaStream_t s) {
+cudaError_t launch_batch_temporal(int prec, const BatchTemporalArgs& a, cudaStream_t s) {
     switch (prec) {
-        case 0: return launch_batch_temporal_f32(a, grid, s);
-        case 1: return launch_batch_temporal_f16(a, grid, s);
-        default: return launch_batch_temporal_bf16(a, grid, s);
+        case 0: return launch_batch_temporal_f32(a, s);
+        case 1: return launch_batch_temporal_f16(a, s);
+        default: return launch_batch_temporal_bf16(a, s);
     }
 }
 

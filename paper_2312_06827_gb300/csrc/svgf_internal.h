@@ -145,9 +145,9 @@ cudaError_t launch_state_import(int prec, int n, const float4* hist_in, const fl
                                 void* hist, void* mom, cudaStream_t s);
 
 // ---- batched frames: descriptors passed by value in the kernel parameters -------------------
-// One persistent launch per stage covers the tiles of up to kMaxBatch images; a block walks the
-// tiles t = blockIdx.x, blockIdx.x + gridDim.x, ...; tile t belongs to the last stream whose
-// tile_base is <= t.  Each stream carries its own Params, so the streams of one launch may be
+// One launch per stage covers the tiles of up to kMaxBatch images; a block walks the tiles
+// t = blockIdx.x, blockIdx.x + gridDim.x, ... (temporal stage: one block a tile); tile t belongs to
+// the last stream whose tile_base is <= t.  Each stream carries its own Params, so the streams of one launch may be
 // different channels (tone mapping, thresholds, rectification, ...) as long as they share the
 // storage precision, the spatial mode and the pass count.  The argument structs stay under the
 // 32 KB kernel-parameter limit (static_asserts below).
@@ -217,7 +217,7 @@ inline void atrous_shape(int shape, int* tx, int* ty) {
     *ty = Y[shape];
 }
 
-cudaError_t launch_batch_temporal(int prec, const BatchTemporalArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_batch_temporal(int prec, const BatchTemporalArgs& a, cudaStream_t s);
 cudaError_t launch_batch_spatial(int prec, const BatchSpatialArgs& a, int grid, cudaStream_t s);
 // mode: 0 = 5x5, 1 = horizontal, 2 = vertical; shape: index into atrous_shape.
 cudaError_t launch_batch_atrous(int prec, int mode, int shape, const BatchAtrousArgs& a, int grid,
