@@ -290,8 +290,9 @@ struct TemporalSmem {
 };
 
 // Resident blocks per SM the temporal kernels' register budget is set for: 4 (64 registers).  With
-// nothing of the gathers held across the barrier the spills are 5 registers; 3 blocks (85 registers,
-// none) measured 242 us a 4K frame against 216.
+// nothing of the gathers held across the barrier the single-frame kernel spills 48 bytes a thread in
+// FP32 storage and 20 in 16 bits (the batched one: svgf_batch.cuh); 3 blocks (85 registers, none)
+// measured 242 us a 4K frame against 216.
 constexpr int kTemporalBlocksPerSM = 4;
 
 // The temporal stage for the TILE_X x TILE_Y tile at (x0, y0) of a W x H image, by a block of
@@ -583,12 +584,11 @@ __device__ __forceinline__ float spatial_weight(const Params& P, float l, float 
 // centre's, so that their roundings are of the size of the deviations: rounded at the size of the
 // luminance, a row's mean cost accuracy wherever the noise is small against it (scattered normals,
 // 1 % noise: 2-norm error of the variance 118 u with the per-tap update, 199 u with absolute row means,
-// 2.3 u so, u = 2^-24).  Bound by instruction issue (79 %
-// with every pixel short): about 52 instructions a tap, where the per-tap update with its
-// division, log1pf and expf took about 95, and a body of one row, where 49 unrolled taps did not
-// fit the instruction cache.  2560x1440 with every pixel short 556 -> 310 us, a steady 1080p
-// frame (some 50 flagged tiles) 21.4 -> 16.3 us.  RC = 0 (the radius from P) keeps West's per-tap
-// update.
+// 2.3 u so, u = 2^-24).  Bound by instruction issue (78 % with every pixel short): about 53 instructions
+// a tap, where the per-tap update with its division, log1pf and expf took about 95, and a body of one
+// row, where 49 unrolled taps did not fit the instruction cache.  2560x1440 with every pixel short
+// 556 -> 313 us (309 with absolute row means), a steady 1080p frame (some 50 flagged tiles)
+// 21.4 -> 16.5 us.  RC = 0 (the radius from P) keeps West's per-tap update.
 template <class S, int RC>
 __device__ __forceinline__ void spatial_variance_tile_r(const Params& P, int W, int H, int x0,
                                                         int y0, const float4* __restrict__ gbuf,

@@ -36,10 +36,13 @@ struct Params {
 // ---- launches that overlap their predecessor's end -------------------------------------------
 // A chained launch (programmatic stream serialization) may start once every block of the launch
 // before it has ended, without waiting for that launch's completion and memory flush; its kernel
-// calls pdl_wait before it touches anything that earlier launches wrote or still read.  pdl_wait
-// returns when the previous launch has completed, which itself waited for its own, so the order of
-// the stream's work is kept.  The first launch of a library call is an ordinary one (pdl_wait then
-// returns at once), so the caller's own work before the call is complete as before.
+// calls pdl_wait before it touches anything that the call's earlier launches wrote or still read.
+// pdl_wait returns when the previous launch has completed, which itself waited for its own, so the
+// order of the stream's work is kept.  The first launch of a library call is an ordinary one (pdl_wait
+// then returns at once), so the caller's own work and the library's earlier calls are complete before
+// any block of the call starts: what they wrote and no launch of this call writes may be read ahead of
+// the wait.  k_conv3x3_tc reads its weights so; no convolution may be chained behind a launch of the
+// same call that writes weights (k_prep_weights ends its calls).
 // Seven launches of a 128x128 frame 59.8 -> 46.7 us, 1080p 490 -> 477 us (5x5) and 437 -> 411 us
 // (separable, 12 launches).  Letting the successor's blocks in while the last wave still runs
 // (griddepcontrol.launch_dependents) was slower for all but the smallest kernels: 504, 425 us.

@@ -375,7 +375,8 @@ __global__ void __launch_bounds__(128 * NG + 64, 2) k_conv3x3_tc(const __grid_co
     uint32_t* tslot = reinterpret_cast<uint32_t*>(fin + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // weights [tap][co][ci] -> per dx the 96 rows (2 - dy) * 32 + co of the B operand, swizzled
-    // like the input rows (64-byte rows for 32 channels, 32-byte rows for 16)
+    // like the input rows (64-byte rows for 32 channels, 32-byte rows for 16).  Read ahead of pdl_wait,
+    // beside the previous launch's end: earlier calls wrote them, and no launch of this one does.
     for (int i = tid; i < 9 * 32 * KG; i += NT) {
         const int kg = i % KG, co = (i / KG) % 32, tap = i / (KG * 32), dy = tap / 3, dx = tap % 3;
         const int r = (2 - dy) * 32 + co;
@@ -1745,10 +1746,12 @@ __global__ void __launch_bounds__(256, 4) k_apply(const float* __restrict__ K, c
 //   the logits' gradient:     dz_j = K_j (gK_j - sum_i K_i gK_i), BF16 [p][32] (zeros past 25).
 // The second application's term is formed here from shared-memory windows of u, c1 and c0 rather
 // than by a kernel of its own that passes 25 FP32 planes (200 B a pixel written and read back)
-// through memory.  Bound by the latency of its weight loads: the weights K_j are read again for the
-// last line (from L1) instead of being kept, and the budget is five blocks a SM (48 registers):
-// 566 us a training step of 16 crops of 256 x 256, against 579, 598 and 644 with four, three and
-// two blocks.  The two kernels before took 53 + 188 us of that step, this one about 115.
+// through memory.  Bound by the latency of its weight loads (12 of 16 waiting warps an issue): the
+// weights K_j are read again for the last line instead of being kept, and the budget is five blocks a
+// SM (48 registers): 566 us a training step of 16 crops of 256 x 256, against 579, 598 and 644 with
+// four, three and two blocks.  The windows of five blocks leave L1 about 30 KB, so the second reads are
+// mostly the L2's (hit rates 12 % in L1, 60 % in L2).  The two kernels before took 53 + 188 us of that
+// step, this one 115.
 __global__ void __launch_bounds__(256, 5) k_bwd_apply(const float* __restrict__ K, const float4* __restrict__ u,
                                                       const float4* __restrict__ c0, const float4* __restrict__ c1,
                                                       const float4* __restrict__ c2, __nv_bfloat16* dz, long np,
