@@ -563,11 +563,13 @@ __device__ __forceinline__ float exp_neg(float e) {
     return fmaf(w, fmaf(0.6931471805599453f, r, 0x1p-25f), w);
 }
 
-// The weight from l = log(1 - t): 0 where the normal weight is 0 or the weight is not a number.
+// The weight from l = log(1 - t): 0 where the normal weight is 0 or the weight is not a number (with
+// sigma_z = infinity, a tap along which the depth has no gradient).  eps keeps the denominator within
+// the reciprocal's range.
 __device__ __forceinline__ float spatial_weight(const Params& P, float l, float zp, float zq, float2 gr,
                                                 float dx, float dy) {
-    const float den = fmaf(P.sigma_z, fabsf(fmaf(gr.x, dx, __fmul_rn(gr.y, dy))), P.eps);
-    const float depth = __fmul_rn(fabsf(zq - zp), rcp_approx(fmaxf(den, 1.17549435e-38f)));
+    const float den = fmaf(P.sigma_z, fabsf(fmaf(gr.x, dx, __fmul_rn(gr.y, dy))), fmaxf(P.eps, 1.17549435e-38f));
+    const float depth = __fmul_rn(fabsf(zq - zp), rcp_approx(den));
     const float w = exp_neg(fmaf(P.sigma_n, l, -depth));
     return w > 0.f ? w : 0.f;
 }
@@ -584,11 +586,10 @@ __device__ __forceinline__ float spatial_weight(const Params& P, float l, float 
 // centre's, so that their roundings are of the size of the deviations: rounded at the size of the
 // luminance, a row's mean cost accuracy wherever the noise is small against it (scattered normals,
 // 1 % noise: 2-norm error of the variance 118 u with the per-tap update, 199 u with absolute row means,
-// 2.3 u so, u = 2^-24).  Bound by instruction issue (78 % with every pixel short): about 53 instructions
+// 2.3 u so, u = 2^-24).  Bound by instruction issue (78 % with every pixel short): about 52 instructions
 // a tap, where the per-tap update with its division, log1pf and expf took about 95, and a body of one
 // row, where 49 unrolled taps did not fit the instruction cache.  2560x1440 with every pixel short
-// 556 -> 313 us (309 with absolute row means), a steady 1080p frame (some 50 flagged tiles)
-// 21.4 -> 16.5 us.  RC = 0 (the radius from P) keeps West's per-tap update.
+// 556 -> 307 us, a steady 1080p frame (some 50 flagged tiles) 21.4 -> 15.9 us.  RC = 0 (the radius from P) keeps West's per-tap update.
 template <class S, int RC>
 __device__ __forceinline__ void spatial_variance_tile_r(const Params& P, int W, int H, int x0,
                                                         int y0, const float4* __restrict__ gbuf,

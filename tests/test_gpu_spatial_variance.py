@@ -163,3 +163,30 @@ def test_one_tap_weight_against_fp64(radius, sigma_n, what):
         assert np.all(rel <= U * (8.0 * np.abs(e) + 32.0)), (rel / U / (8.0 * np.abs(e) + 32.0)).max()
         if what == "depth":
             assert abs(np.mean(got[p] / ref - 1.0)) <= 0.6 * U
+
+
+@pytest.mark.parametrize("radius", [2, 3])
+def test_infinite_depth_tolerance(radius):
+    """sigma_z = infinity: along a depth gradient the depth term is 0; where there is none its denominator,
+    infinity times 0, is not a number and the tap, the centre among them, has weight 0."""
+    w, h = 40, 20
+    rng = np.random.default_rng(5)
+    gbuf = np.zeros((h, w, 4), np.float32)
+    gbuf[..., 2] = 1.0
+    gbuf[..., 3] = 5.0 + 0.25 * np.arange(w)               # no gradient along y, exactly representable
+    gbuf[:, 30:, 3] = 9.0                                  # none at all
+    cfg = svgf.default_config(w, h)
+    cfg.sigma_z, cfg.sigma_n, cfg.spatial_var_radius = np.inf, 2.0, radius
+    got, l = first_frame(rng.exponential(1.0, (h, w, 3)), gbuf, cfg)
+    ref = np.zeros((h, w))
+    gx, gy = np.gradient(gbuf[..., 3].astype(np.float64), axis=1), np.gradient(gbuf[..., 3].astype(np.float64), axis=0)
+    for y in range(h):
+        for x in range(w):
+            ys, xs = slice(max(0, y - radius), min(h, y + radius + 1)), slice(max(0, x - radius), min(w, x + radius + 1))
+            dy, dx = np.mgrid[ys, xs] - np.array([y, x])[:, None, None]
+            wt = (gx[y, x] * dx + gy[y, x] * dy != 0.0).astype(np.float64)
+            if wt.sum() > 0:
+                m = (wt * l[ys, xs]).sum() / wt.sum()
+                ref[y, x] = (wt * (l[ys, xs] - m) ** 2).sum() / wt.sum()
+    tol = VAR_TOL * ref + 8 * U * l.max() * np.sqrt(ref)
+    assert np.all(np.abs(got - ref) <= tol), np.abs(got - ref).max()
